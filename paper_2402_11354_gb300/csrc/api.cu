@@ -468,14 +468,31 @@ peos_status peos_build_codes_permuted(const peos_graph* graph, const peos_matrix
   e = cudaMemcpyAsync(c->A, hA.data(), hA.size() * sizeof(float), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->B, hB.data(), hB.size() * sizeof(float), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->Wt, hW.data(), hW.size() * sizeof(float), cudaMemcpyHostToDevice, s);
+  // the tiled builder reads 16 vectors per coordinate: Wt itself at m = 16, else a zero-padded copy
+  const int pv = codes_padded_vecs();
+  std::vector<float> hW16;
+  if (m < pv) {
+    hW16.assign((size_t)2 * d * pv, 0.0f);
+    for (int t = 0; t < 2 * d; ++t)
+      for (int j = 0; j < m; ++j) hW16[(size_t)t * pv + j] = hW[(size_t)t * m + j];
+  }
+  const size_t w16 = hW16.size() * sizeof(float);
+  const size_t sb = build_codes_scratch_bytes(n, L, m);
+  StreamScratch scratch(s);
+  if (e == cudaSuccess && sb + w16 > 0) e = scratch.alloc(((sb + 255) & ~(size_t)255) + w16);
+  const float* W16 = c->Wt;
+  if (e == cudaSuccess && w16 > 0) {
+    float* dst = reinterpret_cast<float*>(static_cast<char*>(scratch.p) + ((sb + 255) & ~(size_t)255));
+    e = cudaMemcpyAsync(dst, hW16.data(), w16, cudaMemcpyHostToDevice, s);
+    W16 = dst;
+  }
   // node tables first: the code builder reads t(v) for each edge's node term
   if (e == cudaSuccess)
-    e = launch_node_proj(static_cast<const float*>(base->data), n, d, L, m, c->A, c->B, c->perm, c->node_proj,
-                         table_stride(L, m), s);
+    e = launch_node_proj(static_cast<const float*>(base->data), n, d, L, m, c->A, c->B, W16, c->perm, c->node_proj,
+                         table_stride(L, m), c->norms, s);
   if (e == cudaSuccess)
-    e = launch_build_codes(static_cast<const float*>(base->data), n, d, graph->nbrs, R, L, m, c->A, c->B, c->perm,
-                           c->node_proj, table_stride(L, m), c->records, c->rec_stride, s);
-  if (e == cudaSuccess) e = launch_row_norms(static_cast<const float*>(base->data), n, d, c->norms, s);
+    e = launch_build_codes(static_cast<const float*>(base->data), n, d, graph->nbrs, R, L, m, c->A, c->B, W16, c->perm,
+                           c->node_proj, table_stride(L, m), c->records, c->rec_stride, scratch.p, s);
   // the host vectors hA/hB go out of scope: wait for their copies
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {

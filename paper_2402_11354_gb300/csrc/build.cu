@@ -1,11 +1,15 @@
 // Index-time PEOs data (Sec. 4.2 steps (1)-(3)): per edge e = u - v the block
 // norms, ||e||, w_reg, e_res and the L+1 extreme-value codes, and the edge's node
 // term of the statistic (S(t(v)), from v's projection table); per node the
-// projection table.  One CTA per node; all of a node's edges (R <= 64) are staged
-// in shared memory.  With a dimension permutation (Appendix D.1) both work on the
+// projection table.  With a dimension permutation (Appendix D.1) both work on the
 // permuted vectors: coordinate k of a row is read from coordinate perm[k].  Every sum
 // is a plain sequential FP32 sum (compiled with --fmad=false), one thread per output,
 // so the results are reproducible bit for bit.
+//
+// Two forms.  Up to 16 vectors per block (m <= 16, every configuration's m) the tiled
+// kernels: a thread takes whole edges (or rows) and all 16 sums of each, so that a vector
+// element read from shared memory serves several edges.  For larger m one CTA per node
+// with a thread per sum (node_proj_kernel, build_codes_kernel).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -229,6 +233,477 @@ __global__ void row_norms_kernel(const float* __restrict__ X, long long n, int d
   }
 }
 
+// ---- the tiled form, m <= 16 -------------------------------------------------------
+//
+// What bounds it: 2 d m multiplies and as many separate adds per edge (the order of the
+// sums is fixed, so no FMA), 4,096 pairs at d = 128: 3.0 ms of the FP32 pipes for the 13.6M
+// edges of a 1M-node graph (R = 32, 1M x 128).  One thread per dot product (the form for
+// m > 16) reads two operands per multiply and add and computes the empty slots too: 257 ms
+// there.  Here a lane owns two edges and keeps the 16 sums of each in registers: per
+// coordinate the warp reads 64 bytes of vectors (one broadcast) and one coordinate of each
+// edge.  A warp walks its nodes' slots, keeps the valid edges in a queue and works on full
+// tiles of 64, so empty slots cost nothing (13.6 of 32 slots are edges).  Measured: index
+// build of 1M x 128 269 -> 10.6 ms, of 50,000 x 960 (L = 24) 106 -> 5.7 ms.  Issue slots are
+// then 57% busy and the rest waits on the rows' gathers: 16 warps 10.4 ms, 20 warps 9.4, 24
+// warps 9.3 (and slower at d = 960); four edges per lane 12.5, coordinates of the next chunk
+// kept in registers 10.8 (one build alone, before its index is freed).
+constexpr int kTileWarps = 20;     // one CTA per SM
+constexpr int kEdgesPerLane = 2;
+constexpr int kEdgeTile = 32 * kEdgesPerLane;
+constexpr int kRowsPerLane = 2;    // node tables
+constexpr int kRowTile = 32 * kRowsPerLane;
+constexpr int kTileDims = 16;      // coordinates staged at a time
+// row pitch of the staged tile in 16-byte units: odd, so that lanes reading 16 bytes of 32
+// consecutive rows meet no bank conflict
+constexpr int kTilePitch = kTileDims / 4 + 1;
+constexpr int kNodeChunk = 8;      // nodes a warp takes from the work counter at a time
+constexpr int kVecs = 16;          // vectors per block after zero padding
+// the vectors (2 d x 16 floats) sit in shared memory up to this d, else they are read
+// through L1 (every lane reads the same address)
+constexpr int kMaxSmemVecDim = 256;
+
+// acc[j] += w[j] * x for the 16 vectors' element at one coordinate, two roundings each (the
+// packed multiply and add would be fused into one rounding, and measured no faster)
+__device__ __forceinline__ void mac16(float (&acc)[kVecs], const float4 (&w)[kVecs / 4], float x) {
+#pragma unroll
+  for (int q = 0; q < kVecs / 4; ++q) {
+    acc[4 * q] = __fadd_rn(acc[4 * q], __fmul_rn(w[q].x, x));
+    acc[4 * q + 1] = __fadd_rn(acc[4 * q + 1], __fmul_rn(w[q].y, x));
+    acc[4 * q + 2] = __fadd_rn(acc[4 * q + 2], __fmul_rn(w[q].z, x));
+    acc[4 * q + 3] = __fadd_rn(acc[4 * q + 3], __fmul_rn(w[q].w, x));
+  }
+}
+
+// argmax_j |p_j|, lowest j on ties, as best | (sign << 16), sgn(0) = +1; the zero padding
+// past m never exceeds a kept value
+__device__ __forceinline__ int argmax16(const float (&p)[kVecs]) {
+  int best = 0;
+  float bv = fabsf(p[0]), pv = p[0];
+#pragma unroll
+  for (int j = 1; j < kVecs; ++j) {
+    const float ax = fabsf(p[j]);
+    if (ax > bv) {
+      bv = ax;
+      pv = p[j];
+      best = j;
+    }
+  }
+  return best | ((pv >= 0.0f) ? 0 : 1 << 16);
+}
+
+struct TileArgs {
+  const float* X;
+  long long n;
+  int d;
+  int L, m;
+  const float* W;       // 2 d rows of 16 floats: the b_j, then the a^i_j, k-major
+  const int32_t* perm;  // or null
+  float* node_proj;     // node tables: written by the row kernel, read by the edge kernel
+  int proj_stride;
+  // rows
+  float* norms;         // ||v||^2, or null (permuted coordinates: another order of the sum)
+  // edges
+  const int32_t* nbrs;
+  int R;
+  uint8_t* rec;
+  size_t rec_stride;
+  int bits, cpw, nwords;
+  float2* blocks;       // per warp: {squared block norm, code} of the tile's edges, [L][kEdgeTile]
+  int* work;
+};
+
+// The vectors of the CTA in shared memory (or their global copy).
+template <bool WSMEM>
+__device__ __forceinline__ const float4* tile_vectors(const TileArgs& a, float4* s_w) {
+  const float4* g = reinterpret_cast<const float4*>(a.W);
+  if (!WSMEM) return g;
+  for (int i = threadIdx.x; i < 2 * a.d * (kVecs / 4); i += blockDim.x) s_w[i] = __ldg(g + i);
+  __syncthreads();
+  return s_w;
+}
+
+template <bool WSMEM>
+__device__ __forceinline__ void load_vec(const float4* w, int k, float4 (&out)[kVecs / 4]) {
+#pragma unroll
+  for (int q = 0; q < kVecs / 4; ++q) out[q] = WSMEM ? w[(size_t)k * (kVecs / 4) + q] : __ldg(w + (size_t)k * (kVecs / 4) + q);
+}
+
+// four coordinates of a row from c0 (a multiple of 4), through the permutation if there is one
+template <bool PERM>
+__device__ __forceinline__ float4 row4(const float* X, long long row, int d, int c0, const int32_t* perm) {
+  const float* x = X + (size_t)row * d;
+  if (!PERM) return __ldg(reinterpret_cast<const float4*>(x + c0));
+  return make_float4(__ldg(x + __ldg(perm + c0)), __ldg(x + __ldg(perm + c0 + 1)), __ldg(x + __ldg(perm + c0 + 2)),
+                     __ldg(x + __ldg(perm + c0 + 3)));
+}
+
+// One pass over the coordinates of a staged chunk: KU (4, 2 or 1, a divisor of the block
+// length) coordinates of each of the lane's E rows at a time; `flush` runs at block ends.
+template <int E, int KU, bool WSMEM, class X, class Flush>
+__device__ __forceinline__ void tile_walk(const float4* s_e, const float4* w, int cw, int dp, int& kk, int lane,
+                                          float (&acc)[E][kVecs], X&& element, Flush&& flush) {
+  const float* rows = reinterpret_cast<const float*>(s_e);
+#pragma unroll 1
+  for (int k = 0; k < cw; k += KU) {
+    float x[E][KU];
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+      const float* p = rows + (size_t)(r * 32 + lane) * (kTilePitch * 4) + k;
+      if constexpr (KU == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        x[r][0] = v.x;
+        x[r][1] = v.y;
+        x[r][2] = v.z;
+        x[r][3] = v.w;
+      } else if constexpr (KU == 2) {
+        const float2 v = *reinterpret_cast<const float2*>(p);
+        x[r][0] = v.x;
+        x[r][1] = v.y;
+      } else {
+        x[r][0] = *p;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < KU; ++q) {
+      float4 wv[kVecs / 4];
+      load_vec<WSMEM>(w, k + q, wv);
+#pragma unroll
+      for (int r = 0; r < E; ++r) mac16(acc[r], wv, element(r, x[r][q]));
+    }
+    kk += KU;
+    if (kk == dp) {
+      flush();
+      kk = 0;
+    }
+  }
+}
+
+template <int E>
+__device__ __forceinline__ void clear(float (&acc)[E][kVecs]) {
+#pragma unroll
+  for (int r = 0; r < E; ++r)
+#pragma unroll
+    for (int j = 0; j < kVecs; ++j) acc[r][j] = 0.0f;
+}
+
+// Projection table of every row, out[v][c][j], and ||v||^2: a warp takes 64 rows, two per
+// lane; first the a^i (one sum per block), then the b_j (block by block: a partial sum per
+// block of d/L dims, then the partials).
+template <int KU, bool PERM, bool WSMEM>
+__global__ void __launch_bounds__(kTileWarps * 32, 1) node_rows_kernel(TileArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float4* s_w = reinterpret_cast<float4*>(smem_raw);
+  const float4* w = tile_vectors<WSMEM>(a, s_w);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float4* s_e = s_w + (WSMEM ? 2 * a.d * (kVecs / 4) : 0) + (size_t)warp * kRowTile * kTilePitch;
+  const int d = a.d, L = a.L, m = a.m, dp = d / L;
+  const long long tiles = (a.n + kRowTile - 1) / kRowTile;
+  for (long long t = (long long)blockIdx.x * kTileWarps + warp; t < tiles; t += (long long)gridDim.x * kTileWarps) {
+    const long long v0 = t * kRowTile;
+    auto stage = [&](int c0, int c4) {
+      __syncwarp();
+#pragma unroll 4
+      for (int i = lane; i < kRowTile * (kTileDims / 4); i += 32) {
+        const int row = i / (kTileDims / 4), col = i % (kTileDims / 4);
+        if (col < c4 && v0 + row < a.n) s_e[row * kTilePitch + col] = row4<PERM>(a.X, v0 + row, d, c0 + 4 * col, a.perm);
+      }
+      __syncwarp();
+    };
+    auto store = [&](int r, int c, const float (&p)[kVecs]) {
+      const long long v = v0 + r * 32 + lane;
+      if (v >= a.n) return;
+      float* o = a.node_proj + (size_t)v * a.proj_stride + c * m;
+      if (m == kVecs) {
+#pragma unroll
+        for (int q = 0; q < kVecs / 4; ++q)
+          reinterpret_cast<float4*>(o)[q] = make_float4(p[4 * q], p[4 * q + 1], p[4 * q + 2], p[4 * q + 3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < kVecs; ++j)
+          if (j < m) o[j] = p[j];
+      }
+    };
+    float acc[kRowsPerLane][kVecs];
+    float nrm[kRowsPerLane];
+#pragma unroll
+    for (int r = 0; r < kRowsPerLane; ++r) nrm[r] = 0.0f;
+    clear(acc);
+    int kk = 0, c = 1;
+    for (int c0 = 0; c0 < d; c0 += kTileDims) {
+      const int cw = min(kTileDims, d - c0);
+      stage(c0, cw >> 2);
+      tile_walk<kRowsPerLane, KU, WSMEM>(
+          s_e, w + (size_t)(d + c0) * (kVecs / 4), cw, dp, kk, lane, acc,
+          [&](int r, float x) {
+            nrm[r] = nrm[r] + x * x;
+            return x;
+          },
+          [&] {
+#pragma unroll
+            for (int r = 0; r < kRowsPerLane; ++r) store(r, c, acc[r]);
+            clear(acc);
+            ++c;
+          });
+    }
+    if (a.norms) {
+#pragma unroll
+      for (int r = 0; r < kRowsPerLane; ++r)
+        if (v0 + r * 32 + lane < a.n) a.norms[v0 + r * 32 + lane] = nrm[r];
+    }
+    float tot[kRowsPerLane][kVecs];
+    clear(tot);
+    for (int c0 = 0; c0 < d; c0 += kTileDims) {
+      const int cw = min(kTileDims, d - c0);
+      stage(c0, cw >> 2);
+      tile_walk<kRowsPerLane, KU, WSMEM>(
+          s_e, w + (size_t)c0 * (kVecs / 4), cw, dp, kk, lane, acc, [&](int, float x) { return x; },
+          [&] {
+#pragma unroll
+            for (int r = 0; r < kRowsPerLane; ++r)
+#pragma unroll
+              for (int j = 0; j < kVecs; ++j) tot[r][j] = tot[r][j] + acc[r][j];
+            clear(acc);
+          });
+    }
+#pragma unroll
+    for (int r = 0; r < kRowsPerLane; ++r) {
+      store(r, 0, tot[r]);
+      const long long v = v0 + r * 32 + lane;
+      if (v < a.n)
+        for (int e = (L + 1) * m; e < a.proj_stride; ++e) a.node_proj[(size_t)v * a.proj_stride + e] = 0.0f;
+    }
+  }
+}
+
+// Edge records.  Per tile of 128 edges two passes over the coordinates: the a^i sums and
+// the block norms (their codes and squared norms go to `blocks`), then, the block norms'
+// mean being known, the b_j sums of e_res.
+template <int KU, bool PERM, bool WSMEM>
+__global__ void __launch_bounds__(kTileWarps * 32, 1) build_edges_kernel(TileArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float4* s_w = reinterpret_cast<float4*>(smem_raw);
+  const float4* w = tile_vectors<WSMEM>(a, s_w);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kQueue = kEdgeTile + 32;
+  constexpr size_t kWarpBytes = (size_t)kEdgeTile * kTilePitch * 16 + (size_t)kQueue * 12;
+  unsigned char* base =
+      reinterpret_cast<unsigned char*>(s_w + (WSMEM ? 2 * a.d * (kVecs / 4) : 0)) + (size_t)warp * kWarpBytes;
+  float4* s_e = reinterpret_cast<float4*>(base);
+  int32_t* q_u = reinterpret_cast<int32_t*>(base + (size_t)kEdgeTile * kTilePitch * 16);
+  int32_t* q_v = q_u + kQueue;
+  int32_t* q_s = q_v + kQueue;
+  const int d = a.d, L = a.L, m = a.m, dp = d / L, R = a.R;
+  float2* blk = a.blocks + ((size_t)blockIdx.x * kTileWarps + warp) * L * kEdgeTile;
+  const size_t ids_end = rec_ids_offset(R) + 4 * (size_t)R, codes_at = rec_codes_offset(R);
+  const size_t used = codes_at + 8 * (size_t)a.nwords * R;
+  const int gap4 = (int)(codes_at - ids_end) / 4, pad4 = (int)(a.rec_stride - used) / 4;
+
+  long long v0 = 0;       // the chunk's first node
+  int slots = 0, at = 0;  // its slots, and how many are queued or written
+  bool more = true;
+  int queued = 0;
+  for (;;) {
+    // ---- fill the queue: the slots' ids go to the records, empty slots are zeroed
+    while (queued < kEdgeTile && more) {
+      if (at >= slots) {
+        int c = 0;
+        if (lane == 0) c = atomicAdd(a.work, 1);
+        v0 = (long long)__shfl_sync(kFull, c, 0) * kNodeChunk;
+        if (v0 >= a.n) {
+          more = false;
+          break;
+        }
+        const int nn = (int)min((long long)kNodeChunk, a.n - v0);
+        slots = nn * R;
+        at = 0;
+        for (int t = lane; t < nn * (gap4 + pad4); t += 32) {
+          const int v = t / (gap4 + pad4), b = t - v * (gap4 + pad4);
+          uint8_t* r = a.rec + (size_t)(v0 + v) * a.rec_stride;
+          *reinterpret_cast<uint32_t*>(b < gap4 ? r + ids_end + 4 * b : r + used + 4 * (b - gap4)) = 0u;
+        }
+      }
+      const int t = at + lane;
+      int32_t u = -1, s = 0;
+      long long v = v0;
+      if (t < slots) {
+        u = __ldg(a.nbrs + (size_t)v0 * R + t);
+        const int lv = t / R;
+        v = v0 + lv;
+        s = t - lv * R;
+        uint8_t* r = a.rec + (size_t)v * a.rec_stride;
+        reinterpret_cast<int32_t*>(r + rec_ids_offset(R))[s] = u;
+        if (u < 0) {
+          reinterpret_cast<float4*>(r)[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int k = 0; k < a.nwords; ++k) reinterpret_cast<uint64_t*>(r + codes_at)[(size_t)k * R + s] = 0;
+        }
+      }
+      const unsigned have = __ballot_sync(kFull, u >= 0);
+      if (u >= 0) {
+        const int p = queued + __popc(have & ((1u << lane) - 1u));
+        q_u[p] = u;
+        q_v[p] = (int32_t)v;
+        q_s[p] = s;
+      }
+      queued += __popc(have);
+      at += 32;
+    }
+    __syncwarp();
+    const int cnt = min(queued, kEdgeTile);
+    if (cnt == 0) break;
+
+    auto stage = [&](int c0) {
+      const int c4 = min(kTileDims, d - c0) >> 2;
+      __syncwarp();
+#pragma unroll 4
+      for (int i = lane; i < kEdgeTile * (kTileDims / 4); i += 32) {
+        const int e = i / (kTileDims / 4), col = i % (kTileDims / 4);
+        if (col < c4 && e < cnt) {
+          const float4 x = row4<PERM>(a.X, q_u[e], d, c0 + 4 * col, a.perm);
+          const float4 y = row4<PERM>(a.X, q_v[e], d, c0 + 4 * col, a.perm);
+          s_e[e * kTilePitch + col] = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
+        }
+      }
+      __syncwarp();
+    };
+
+    // ---- pass 1: block norms and the codes e[1..L]
+    float acc[kEdgesPerLane][kVecs];
+    clear(acc);
+    int kk = 0, c = 0;
+    {
+      float n2[kEdgesPerLane];
+#pragma unroll
+      for (int r = 0; r < kEdgesPerLane; ++r) n2[r] = 0.0f;
+      for (int c0 = 0; c0 < d; c0 += kTileDims) {
+        const int cw = min(kTileDims, d - c0);
+        stage(c0);
+        tile_walk<kEdgesPerLane, KU, WSMEM>(
+            s_e, w + (size_t)(d + c0) * (kVecs / 4), cw, dp, kk, lane, acc,
+            [&](int r, float x) {
+              n2[r] = n2[r] + x * x;
+              return x;
+            },
+            [&] {
+#pragma unroll
+              for (int r = 0; r < kEdgesPerLane; ++r) {
+                blk[(size_t)c * kEdgeTile + r * 32 + lane] = make_float2(n2[r], __int_as_float(argmax16(acc[r])));
+                n2[r] = 0.0f;
+              }
+              clear(acc);
+              ++c;
+            });
+      }
+    }
+    // ---- ||e||, the weights, the packed codes and the regular part of the node term
+    float mean[kEdgesPerLane];
+#pragma unroll
+    for (int r = 0; r < kEdgesPerLane; ++r) {
+      const int e = r * 32 + lane;
+      mean[r] = 0.0f;
+      if (e >= cnt) continue;
+      float tot2 = 0.0f, sum = 0.0f;
+#pragma unroll 4
+      for (int i = 0; i < L; ++i) {
+        const float b2 = blk[(size_t)i * kEdgeTile + e].x;
+        tot2 = tot2 + b2;
+        sum = sum + sqrtf(b2);
+      }
+      const float norm = sqrtf(tot2);
+      float wr = 1.0f, cr = 0.0f;
+      if (norm != 0.0f) {
+        wr = sum / (sqrtf((float)L) * norm);
+        if (wr > 1.0f) wr = 1.0f;
+        cr = sqrtf((float)L) * sqrtf(fmaxf(0.0f, 1.0f - wr * wr));
+        mean[r] = sum / (float)L;
+      }
+      uint8_t* rec = a.rec + (size_t)q_v[e] * a.rec_stride;
+      uint64_t* cwords = reinterpret_cast<uint64_t*>(rec + codes_at) + q_s[e];
+      const float* tv = a.node_proj + (size_t)q_v[e] * a.proj_stride;
+      float h1 = 0.0f;
+      uint64_t word = 0;
+      int k = 1, wi = 0;
+      for (int i0 = 0; i0 < L; i0 += 4) {
+        int sel[4];
+        float val[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          // a degenerate edge gets code +1 everywhere
+          sel[q] = (i0 + q < L && norm != 0.0f) ? __float_as_int(blk[(size_t)(i0 + q) * kEdgeTile + e].y) : 0;
+          val[q] = i0 + q < L ? __ldg(tv + (i0 + q + 1) * m + (sel[q] & 0xffff)) : 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (i0 + q >= L) break;
+          h1 = h1 + ((sel[q] >> 16) ? -val[q] : val[q]);
+          word |= ((uint64_t)(sel[q] & 0xffff) | ((uint64_t)(sel[q] >> 16) << (a.bits - 1))) << (k * a.bits);
+          if (++k == a.cpw) {
+            cwords[(size_t)wi * R] = word;
+            word = 0;
+            k = 0;
+            ++wi;
+          }
+        }
+      }
+      if (k > 0) cwords[(size_t)wi * R] = word;
+      reinterpret_cast<float4*>(rec)[q_s[e]] = make_float4(norm, wr, cr, h1);  // h1 becomes the node term below
+    }
+    // ---- pass 2: e_res = e - e_reg (block i scaled by 1 - mean(||e_k||) / ||e_i||) and e[0]
+    {
+      float coef[kEdgesPerLane];
+      auto scale = [&](int i) {
+#pragma unroll
+        for (int r = 0; r < kEdgesPerLane; ++r) {
+          const float b = sqrtf(blk[(size_t)i * kEdgeTile + r * 32 + lane].x);
+          coef[r] = (b > 0.0f) ? (1.0f - mean[r] / b) : 0.0f;
+        }
+      };
+      scale(0);
+      c = 0;
+      for (int c0 = 0; c0 < d; c0 += kTileDims) {
+        const int cw = min(kTileDims, d - c0);
+        stage(c0);
+        tile_walk<kEdgesPerLane, KU, WSMEM>(
+            s_e, w + (size_t)c0 * (kVecs / 4), cw, dp, kk, lane, acc, [&](int r, float x) { return x * coef[r]; },
+            [&] {
+              if (++c < L) scale(c);
+            });
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kEdgesPerLane; ++r) {
+      const int e = r * 32 + lane;
+      if (e < cnt) {
+        uint8_t* rec = a.rec + (size_t)q_v[e] * a.rec_stride;
+        float4* sc = reinterpret_cast<float4*>(rec) + q_s[e];
+        uint64_t* cwords = reinterpret_cast<uint64_t*>(rec + codes_at) + q_s[e];
+        float4 f = *sc;
+        const int sel = f.x == 0.0f ? 0 : argmax16(acc[r]);
+        const float v0f = __ldg(a.node_proj + (size_t)q_v[e] * a.proj_stride + (sel & 0xffff));
+        const float h2 = (sel >> 16) ? -v0f : v0f;
+        f.w = f.y * f.w + f.z * h2;
+        *sc = f;
+        *cwords = *cwords | (uint64_t)(sel & 0xffff) | ((uint64_t)(sel >> 16) << (a.bits - 1));
+      }
+    }
+    // ---- the queue's rest moves to the front
+    const int rest = queued - cnt;
+    int32_t ru = 0, rv = 0, rs = 0;
+    __syncwarp();
+    if (lane < rest) {
+      ru = q_u[cnt + lane];
+      rv = q_v[cnt + lane];
+      rs = q_s[cnt + lane];
+    }
+    __syncwarp();
+    if (lane < rest) {
+      q_u[lane] = ru;
+      q_v[lane] = rv;
+      q_s[lane] = rs;
+    }
+    queued = rest;
+  }
+}
+
 int num_sms() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 1;
@@ -356,10 +831,76 @@ cudaError_t launch_compact_records(const uint8_t* src, size_t src_stride, int64_
   return cudaGetLastError();
 }
 
+namespace {
+
+// The tiled kernels' variant for the block length: 4, 2 or 1 coordinates per step, rows
+// read through a permutation or not, the vectors in shared memory or not.
+template <bool EDGES, int KU, bool PERM, bool WSMEM>
+cudaError_t launch_tile(const TileArgs& a, int grid, cudaStream_t st) {
+  const void* fn = EDGES ? (const void*)build_edges_kernel<KU, PERM, WSMEM> : (const void*)node_rows_kernel<KU, PERM, WSMEM>;
+  const size_t per_warp = EDGES ? (size_t)kEdgeTile * kTilePitch * 16 + (size_t)(kEdgeTile + 32) * 12
+                                : (size_t)kRowTile * kTilePitch * 16;
+  const size_t smem = (WSMEM ? (size_t)2 * a.d * kVecs * sizeof(float) : 0) + per_warp * kTileWarps;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  TileArgs copy = a;
+  void* args[] = {&copy};
+  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kTileWarps * 32), args, smem, st);
+}
+template <bool EDGES, int KU>
+cudaError_t launch_tile_ku(const TileArgs& a, int grid, cudaStream_t st) {
+  const bool ws = a.d <= kMaxSmemVecDim;
+  if (a.perm) return ws ? launch_tile<EDGES, KU, true, true>(a, grid, st) : launch_tile<EDGES, KU, true, false>(a, grid, st);
+  return ws ? launch_tile<EDGES, KU, false, true>(a, grid, st) : launch_tile<EDGES, KU, false, false>(a, grid, st);
+}
+template <bool EDGES>
+cudaError_t launch_tile_any(const TileArgs& a, int grid, cudaStream_t st) {
+  const int dp = a.d / a.L;
+  return dp % 4 == 0   ? launch_tile_ku<EDGES, 4>(a, grid, st)
+         : dp % 2 == 0 ? launch_tile_ku<EDGES, 2>(a, grid, st)
+                       : launch_tile_ku<EDGES, 1>(a, grid, st);
+}
+
+int edges_grid(int64_t n) { return (int)std::min<int64_t>(num_sms(), (n + kNodeChunk - 1) / kNodeChunk); }
+
+}  // namespace
+
+int codes_padded_vecs() { return kVecs; }
+
+size_t build_codes_scratch_bytes(int64_t n, int L, int m) {
+  if (m > kVecs || n <= 0) return 0;
+  return 256 + (size_t)edges_grid(n) * kTileWarps * L * kEdgeTile * sizeof(float2);
+}
+
 cudaError_t launch_build_codes(const float* X, int64_t n, int d, const int32_t* nbrs, int R, int L, int m,
-                               const float* A, const float* B, const int32_t* perm, const float* node_proj,
-                               int proj_stride, uint8_t* rec, size_t rec_stride, cudaStream_t st) {
+                               const float* A, const float* B, const float* W16, const int32_t* perm,
+                               const float* node_proj, int proj_stride, uint8_t* rec, size_t rec_stride,
+                               void* scratch, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
+  if (m <= kVecs) {
+    cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    TileArgs a{};
+    a.X = X;
+    a.n = n;
+    a.d = d;
+    a.L = L;
+    a.m = m;
+    a.W = W16;
+    a.perm = perm;
+    a.node_proj = const_cast<float*>(node_proj);
+    a.proj_stride = proj_stride;
+    a.nbrs = nbrs;
+    a.R = R;
+    a.rec = rec;
+    a.rec_stride = rec_stride;
+    a.bits = code_bits(m);
+    a.cpw = codes_per_word(m);
+    a.nwords = code_words(L, m);
+    a.work = static_cast<int*>(scratch);
+    a.blocks = reinterpret_cast<float2*>(static_cast<unsigned char*>(scratch) + 256);
+    return launch_tile_any<true>(a, edges_grid(n), st);
+  }
   const size_t smem = sizeof(float) * ((size_t)R * d + 2 * (size_t)R * L + 4 * (size_t)R +
                                        (size_t)R * (L + 1) * m) +
                       sizeof(int32_t) * ((size_t)R + (size_t)R * (L + 1)) + sizeof(float) * (size_t)(L + 1) * m;
@@ -378,14 +919,33 @@ cudaError_t launch_build_codes(const float* X, int64_t n, int d, const int32_t* 
 }
 
 cudaError_t launch_node_proj(const float* X, int64_t n, int d, int L, int m, const float* A, const float* B,
-                             const int32_t* perm, float* out, int out_stride, cudaStream_t st) {
+                             const float* W16, const int32_t* perm, float* out, int out_stride, float* norms,
+                             cudaStream_t st) {
   if (n == 0) return cudaSuccess;
+  if (m <= kVecs) {
+    TileArgs a{};
+    a.X = X;
+    a.n = n;
+    a.d = d;
+    a.L = L;
+    a.m = m;
+    a.W = W16;
+    a.perm = perm;
+    a.node_proj = out;
+    a.proj_stride = out_stride;
+    a.norms = perm ? nullptr : norms;  // the norm sums the stored order of the coordinates
+    const int64_t ctas = (n + (int64_t)kRowTile * kTileWarps - 1) / ((int64_t)kRowTile * kTileWarps);
+    cudaError_t e = launch_tile_any<false>(a, (int)std::min<int64_t>(num_sms(), ctas), st);
+    if (e != cudaSuccess || !perm) return e;
+    return launch_row_norms(X, n, d, norms, st);
+  }
   const long long total = n * (long long)out_stride;
   long long grid = (total + 255) / 256;
   const long long cap = (long long)num_sms() * 16;
   if (grid > cap) grid = cap;
   node_proj_kernel<<<(unsigned)grid, 256, 0, st>>>(X, n, d, L, m, A, B, perm, out, out_stride);
-  return cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? launch_row_norms(X, n, d, norms, st) : e;
 }
 
 cudaError_t launch_row_norms(const float* X, int64_t n, int d, float* norms, cudaStream_t st) {
