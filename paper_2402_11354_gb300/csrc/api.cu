@@ -1065,6 +1065,12 @@ peos_status peos_selftest_bounded_wait(int64_t limit_us, int32_t* gave_up, void*
   return PEOS_OK;
 }
 
+// Bases from this size on take the tensor-core scores first (d = 100, k = 10, 1 / 2,000
+// queries, FFMA alone against scores: 2,048 rows 199 / 246 us against 114 / 172; 16,384 rows
+// 1187 / 1366 against 123 / 324; 300,000 rows 1.5 / 6.8 ms against 0.25 / 0.94; below, the
+// six launches cost what one does).
+static constexpr int64_t kKnnExactMinRows = 2048;
+
 peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* queries, int32_t k, int32_t* ids_out,
                                 float* dists_out, void* stream) {
   NvtxRange nvtx_range("peos.knn");
@@ -1084,14 +1090,34 @@ peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* quer
   int64_t slice = (int64_t)((size_t)1 << 30) / (int64_t)per_query;
   slice = slice < 32 ? 32 : slice - slice % 32;
   if (slice > queries->n) slice = queries->n;
+  const size_t lists = (knn_scratch_bytes(base->n, slice, k) + 255) & ~(size_t)255;
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  size_t exact = base->n >= kKnnExactMinRows && base->n <= 0x7fffffffLL
+                     ? knn_exact_scratch_bytes(base->n, slice, base->d, k, sms)
+                     : 0;
   StreamScratch scratch(s);
-  cudaError_t e = scratch.alloc(knn_scratch_bytes(base->n, slice, k));
+  cudaError_t e = scratch.alloc(lists + exact);
+  if (e == cudaErrorMemoryAllocation && exact) {  // the converted base does not fit: FFMA alone
+    (void)cudaGetLastError();
+    exact = 0;
+    e = scratch.alloc(lists);
+  }
   if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync knn scratch");
+  const float* X = static_cast<const float*>(base->data);
   const float* Q = static_cast<const float*>(queries->data);
+  void* tc = static_cast<char*>(scratch.p) + lists;
   for (int64_t q0 = 0; q0 < queries->n; q0 += slice) {
     const int64_t nq = queries->n - q0 < slice ? queries->n - q0 : slice;
-    e = launch_knn(static_cast<const float*>(base->data), base->n, base->d, Q + (size_t)q0 * base->d, nq, k,
-                   ids_out + (size_t)q0 * k, dists_out + (size_t)q0 * k, scratch.p, s);
+    int32_t* ids = ids_out + (size_t)q0 * k;
+    float* dists = dists_out + (size_t)q0 * k;
+    const size_t need = exact ? knn_exact_scratch_bytes(base->n, nq, base->d, k, sms) : 0;
+    e = cudaErrorNotSupported;
+    if (need > 0 && need <= exact)
+      e = launch_knn_exact(X, base->n, base->d, Q + (size_t)q0 * base->d, nq, k, ids, dists, tc, scratch.p, sms, s);
+    if (e == cudaErrorNotSupported)  // also where tensor maps are not available
+      e = launch_knn(X, base->n, base->d, Q + (size_t)q0 * base->d, nq, k, ids, dists, scratch.p, s);
     if (e != cudaSuccess) return cuda_error(e, "knn launch");
   }
   return PEOS_OK;

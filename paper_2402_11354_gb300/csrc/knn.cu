@@ -7,6 +7,9 @@
 // its queries' k best (dist, id) keys of the chunk sorted in shared memory and
 // writes them to scratch [nq][chunks][k].
 // Pass 2: one warp per query merges its chunks' lists into the final k.
+//
+// With a query list (`qlist`, its length in device memory) the same for the listed queries
+// only: the ones whose result the tensor-core form (knn_tc.cu) could not prove.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -48,7 +51,11 @@ __device__ __forceinline__ void warp_list_insert(uint64_t* lst, int k, uint64_t 
 
 __global__ void __launch_bounds__(kThreads) knn_chunk_kernel(const float* __restrict__ X, long long n, int d,
                                                              const float* __restrict__ Q, long long nq, int k,
-                                                             int nchunks, uint64_t* __restrict__ part) {
+                                                             int nchunks, uint64_t* __restrict__ part,
+                                                             const int32_t* __restrict__ qlist,
+                                                             const int* __restrict__ qcount) {
+  if (qlist) nq = *qcount;
+  if ((long long)blockIdx.x * kQT >= nq) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* qs = reinterpret_cast<float*>(smem_raw);          // [kQT][kDK]
   float* xs = qs + kQT * kDK;                               // [kDK][kPT]
@@ -72,7 +79,10 @@ __global__ void __launch_bounds__(kThreads) knn_chunk_kernel(const float* __rest
       for (int i = tid; i < kQT * (kDK / 4); i += kThreads) {
         const int qq = i / (kDK / 4), c4 = i - qq * (kDK / 4);
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (q0 + qq < nq && c4 * 4 < dk) v = *reinterpret_cast<const float4*>(Q + (size_t)(q0 + qq) * d + k0 + c4 * 4);
+        if (q0 + qq < nq && c4 * 4 < dk) {
+          const long long row = qlist ? qlist[q0 + qq] : q0 + qq;
+          v = *reinterpret_cast<const float4*>(Q + (size_t)row * d + k0 + c4 * 4);
+        }
         *reinterpret_cast<float4*>(qs + qq * kDK + c4 * 4) = v;
       }
       for (int i = tid; i < kPT * (kDK / 4); i += kThreads) {
@@ -125,7 +135,9 @@ __global__ void __launch_bounds__(kThreads) knn_chunk_kernel(const float* __rest
 }
 
 __global__ void knn_merge_kernel(const uint64_t* __restrict__ part, long long nq, int k, int nchunks,
-                                 int32_t* __restrict__ ids_out, float* __restrict__ dists_out) {
+                                 int32_t* __restrict__ ids_out, float* __restrict__ dists_out,
+                                 const int32_t* __restrict__ qlist, const int* __restrict__ qcount) {
+  if (qlist) nq = *qcount;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   uint64_t* lst = reinterpret_cast<uint64_t*>(smem_raw) + (size_t)warp * k;
@@ -147,8 +159,9 @@ __global__ void knn_merge_kernel(const uint64_t* __restrict__ part, long long nq
     }
     for (int i = lane; i < k; i += 32) {
       const uint64_t key = lst[i];
-      ids_out[(size_t)q * k + i] = key == kNoKey ? -1 : key_id(key);
-      dists_out[(size_t)q * k + i] = key == kNoKey ? INFINITY : key_dist(key);
+      const size_t o = (size_t)(qlist ? qlist[q] : q) * k + i;
+      ids_out[o] = key == kNoKey ? -1 : key_id(key);
+      dists_out[o] = key == kNoKey ? INFINITY : key_dist(key);
     }
     __syncwarp();
   }
@@ -162,7 +175,7 @@ size_t knn_scratch_bytes(int64_t n, int64_t nq, int k) {
 }
 
 cudaError_t launch_knn(const float* X, int64_t n, int d, const float* Q, int64_t nq, int k, int32_t* ids_out,
-                       float* dists_out, void* scratch, cudaStream_t st) {
+                       float* dists_out, void* scratch, cudaStream_t st, const int32_t* qlist, const int* qcount) {
   if (nq == 0) return cudaSuccess;
   const int nchunks = (int)((n + kChunk - 1) / kChunk);
   uint64_t* part = static_cast<uint64_t*>(scratch);
@@ -170,7 +183,7 @@ cudaError_t launch_knn(const float* X, int64_t n, int d, const float* Q, int64_t
   cudaError_t e = cudaFuncSetAttribute(knn_chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
   if (e != cudaSuccess) return e;
   dim3 grid1((unsigned)((nq + kQT - 1) / kQT), (unsigned)nchunks);
-  knn_chunk_kernel<<<grid1, kThreads, smem1, st>>>(X, n, d, Q, nq, k, nchunks, part);
+  knn_chunk_kernel<<<grid1, kThreads, smem1, st>>>(X, n, d, Q, nq, k, nchunks, part, qlist, qcount);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int wpb = 4;
@@ -179,7 +192,8 @@ cudaError_t launch_knn(const float* X, int64_t n, int d, const float* Q, int64_t
   if (e != cudaSuccess) return e;
   long long g2 = (nq + wpb - 1) / wpb;
   if (g2 > 65535) g2 = 65535;
-  knn_merge_kernel<<<(unsigned)g2, wpb * 32, smem2, st>>>(part, nq, k, nchunks, ids_out, dists_out);
+  knn_merge_kernel<<<(unsigned)g2, wpb * 32, smem2, st>>>(part, nq, k, nchunks, ids_out, dists_out, qlist,
+                                                             qcount);
   return cudaGetLastError();
 }
 

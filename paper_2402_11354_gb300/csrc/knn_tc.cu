@@ -1,25 +1,34 @@
-// Brute-force K-NN on the tensor cores (sm_103a tcgen05): the ground truth of the recall
-// metric for large bases.
+// Brute-force K-NN on the tensor cores (sm_103a tcgen05): graph candidates and ground truth
+// for large bases, in two precisions of the scores.
 //
 //   1. convert: base and queries to BF16 rows (zero-padded to a multiple of 64 elements),
-//      and ||x||^2 of every base row in FP32;
-//   2. candidates: per CTA (one per SM), a tile of 128 queries against one slice of the
-//      base, the number of slices chosen by a cost model of waves, tiles and insertions.  A TMA warp brings
-//      128 x 64 query and 256 x 64 base tiles (128-byte swizzled, K-major) into a ring of
-//      2-4 shared-memory stages behind mbarriers; an MMA warp issues tcgen05.mma (BF16 in,
-//      FP32 accumulate in tensor memory, M = 128, N = 256, K = 16 per instruction) into one
-//      of two accumulators; four epilogue warps read the other accumulator with
-//      tcgen05.ld, one query row per thread, screen 32 scores ||x||^2 - 2 q.x at a time
-//      against the row's worst kept score (q's own norm does not change the order) and
-//      insert the few that may enter the row's best `cand`, kept as a max-heap in shared
-//      memory (the root is the worst kept key; an insertion replaces it and sifts down);
-//   3. finalize: one warp per query takes the candidates of every slice, computes their
-//      exact FP32 squared distances from the FP32 rows (sequential over the dimensions)
-//      and keeps the k smallest by (dist, id).
+//      and ||x||^2 of every base row in FP32.  The precise form keeps each value as the sum
+//      of two BF16 terms, hi and lo, in a row of twice the length.
+//   2. candidates: one CTA per SM takes an equal, contiguous share of the (128 queries x 256
+//      base rows) tiles, query tile by query tile; a query tile that spans CTAs has one
+//      candidate list per CTA (a segment).  A TMA warp brings 128 x 64 query and 256 x 64 base
+//      chunks (128-byte swizzled, K-major) through a ring of shared-memory stages behind
+//      mbarriers (the query chunks stay resident where they fit); an MMA warp issues
+//      tcgen05.mma (BF16 in, FP32 accumulate in tensor memory, M = 128, N = 256, K = 16 per
+//      instruction) into one of two accumulators, in the precise form for the products hi hi,
+//      lo hi and hi lo; four epilogue warps read the other accumulator with tcgen05.ld, one
+//      query row per thread, and keep the row's best `cand` scores ||x||^2 - 2 q.x (q's own
+//      norm does not change the order) in a max-heap in shared memory.  Scores below the
+//      heap's worst wait in a short per-row buffer; when a row's buffer is nearly full all
+//      rows empty theirs side by side.
+//   3. finalize: the candidates of every segment sorted by score; those that may be among
+//      the k nearest (score within twice the error bound of the k-th) get their exact FP32
+//      squared distance (sequential over the dimensions), and the k smallest by (dist, id)
+//      are the result.
 // On integer-valued data below 256 (SIFT-shaped) the BF16 products and their FP32 sums
-// are exact, so the candidates are exactly the best rows of each slice.  Otherwise the
+// are exact, so the candidates are exactly the best rows of each segment.  Otherwise the
 // BF16 rounding only reorders near-ties, which the slack of `cand` over k absorbs; the
 // final distances are always exact FP32.
+//
+// The precise form proves its result: a row left out of a full list scored no better than
+// that list's worst, so with the score's error bound its distance is known to be above
+// the k-th found, or the query is handed on to the FFMA kernel (knn.cu).  Non-finite or
+// vanishing norms and a CTA that gave up waiting hand every query on.
 //
 // Every wait on an mbarrier is bounded: after kWaitLimitNs of the global timer (or
 // kMaxPolls polls, whichever comes first) the CTA records an error and stops issuing work
@@ -28,7 +37,9 @@
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <float.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "device.cuh"
@@ -41,15 +52,17 @@ constexpr int kTcM = 128;      // queries per tile: accumulator rows = tensor-me
 constexpr int kTcN = 256;      // base rows per tile: accumulator columns
 constexpr int kTcK = 64;       // elements per stage: one 128-byte swizzle atom of BF16
 constexpr int kMaxStages = 4;
-constexpr int kEpiWarps = 4;                       // one per quarter of the tensor-memory lanes
-constexpr int kEpiThreads = kEpiWarps * 32;        // = kTcM: one accumulator row per thread
-constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
-constexpr int kTcThreads = (kEpiWarps + 2) * 32;
+constexpr int kRows = kTcM;                        // candidate lists per CTA: one per accumulator row
 constexpr int kAccCols = 2 * kTcN;                 // two accumulators: all 512 tensor-memory columns
 constexpr long long kWaitLimitNs = 2000000000ll;  // 2 s: no wait of a healthy launch comes near it
 constexpr long long kMaxPolls = 1ll << 26;
-constexpr int kMaxK = 96;          // k this path serves (candidates per slice: k + 16)
-constexpr int kMaxCandTotal = 2048;  // candidates per query over all slices (finalize's shared memory)
+constexpr int kMaxK = 96;          // k peos_knn_tensor serves (candidates per segment: k + 16)
+constexpr int kMaxCandTotal = 4096;  // candidates per query over all segments (finalize's shared memory)
+// Columns screened together, and scores a row buffers before they enter its heap (at least a
+// group): 16 and 20 per warp where 8 epilogue warps' buffers fit in shared memory beside the
+// lists, 8 and 12 with 4 warps (long lists).
+__host__ __device__ constexpr int group_cols(int ew) { return ew == 8 ? 16 : 8; }
+__host__ __device__ constexpr int pend_slots(int ew) { return ew == 8 ? 20 : 12; }
 
 constexpr int kABytes = kTcM * kTcK * 2;  // 16 KB
 constexpr int kBBytes = kTcN * kTcK * 2;  // 32 KB
@@ -142,42 +155,83 @@ __device__ __forceinline__ uint32_t ordered(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// the score of a candidate key (inverse of ordered on the high word); +inf for an empty
-// slot, so that every finite score may enter a list that is not full
+// the score of a candidate key (inverse of ordered on the high word); the largest finite
+// value for an empty slot, so that every finite score may enter a list that is not full and
+// +inf (a column past the base) never does
 __device__ __forceinline__ float key_score(uint64_t key) {
-  if (key == kNoKey) return INFINITY;
+  if (key == kNoKey) return FLT_MAX;
   const uint32_t o = (uint32_t)(key >> 32);
   return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// One warp per row, four elements per lane.  LO: the rounding errors' own BF16 values follow
+// the row's hi terms.  norm2: FP32 squared norms (base rows); xmax: the largest of them, as
+// its bits (a NaN's bits are larger than any number's).
+template <bool LO>
 __global__ void convert_bf16_kernel(const float* __restrict__ X, long long n, int d, int pitch,
-                                    __nv_bfloat16* __restrict__ out, float* __restrict__ norm2) {
+                                    __nv_bfloat16* __restrict__ out, float* __restrict__ norm2,
+                                    unsigned* __restrict__ xmax) {
   const int lane = threadIdx.x & 31;
   const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+  const size_t row = (size_t)pitch * (LO ? 2 : 1);
+  unsigned most = 0;
   for (long long r = w0; r < n; r += nw) {
     float s = 0.0f;
-    for (int k = lane; k < pitch; k += 32) {
-      const float v = k < d ? X[(size_t)r * d + k] : 0.0f;
-      out[(size_t)r * pitch + k] = __float2bfloat16_rn(v);
-      s += v * v;
+    for (int k = 4 * lane; k < pitch; k += 128) {
+      const float4 v = k < d ? __ldg(reinterpret_cast<const float4*>(X + (size_t)r * d + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const uint2 h = make_uint2(bf16_pair(v.x, v.y), bf16_pair(v.z, v.w));
+      *reinterpret_cast<uint2*>(out + (size_t)r * row + k) = h;
+      if (LO) {
+        const float4 f = make_float4(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xffff0000u),
+                                     __uint_as_float(h.y << 16), __uint_as_float(h.y & 0xffff0000u));
+        *reinterpret_cast<uint2*>(out + (size_t)r * row + pitch + k) =
+            make_uint2(bf16_pair(v.x - f.x, v.y - f.y), bf16_pair(v.z - f.z, v.w - f.w));
+      }
+      s += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
     }
     if (norm2) {
       s = warp_sum(s);
       if (lane == 0) norm2[r] = s;
+      most = max(most, __float_as_uint(s));
     }
   }
+  if (norm2 && lane == 0 && most) atomicMax(xmax, most);
 }
+
+// The tiles of one launch: qt x bt, handed out in equal contiguous shares to G CTAs.
+struct TcShare {
+  long long units;  // qt * bt
+  int bt, G;
+  __host__ __device__ long long start(int c) const { return units * c / G; }
+  // the CTA whose share holds unit u
+  __host__ __device__ int cta_of(long long u) const { return (int)(((u + 1) * G - 1) / units); }
+  // most CTAs that share one query tile
+  __host__ int max_segments() const {
+    int most = 1;
+    for (long long q = 0; q * bt < units; ++q) {
+      const int s = cta_of(q * bt + bt - 1) - cta_of(q * bt) + 1;
+      if (s > most) most = s;
+    }
+    return most;
+  }
+};
 
 struct TcArgs {
   const float* xnorm;
   long long n, nq;
+  TcShare share;
   int kchunks;       // pitch / 64
-  int cand;          // candidates kept per query per slice
-  long long slice;   // base rows per slice
-  int nslice;
+  int cand;          // candidates kept per query per segment
   int stages;        // shared-memory ring depth (2..kMaxStages)
-  uint64_t* out;     // [nq][nslice][cand] (ordered(approx) << 32 | id)
+  uint32_t row0;     // id of the launch's first base row
+  int nseg, seg0;    // segments per query in `out`, and the launch's first
+  uint64_t* out;     // [nq][nseg][cand] (ordered(approx) << 32 | id), prefilled with kNoKey
   int* err;
 };
 
@@ -185,50 +239,205 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory"); }
+// the epilogue warps that serve one quarter of the rows (one warp, or two)
+template <int EW>
+__device__ __forceinline__ void quarter_sync(int quarter) {
+  if (EW == 4) __syncwarp();
+  else asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");
+}
 
-// Warp-specialised: warps 0-3 read the accumulator (each its quarter of the tensor-memory
-// lanes, one query row per thread) and keep the candidates; warp 4 issues the TMA loads
-// into a ring of `stages` shared-memory stages; warp 5 issues the MMAs into one of two
-// accumulators (512 tensor-memory columns), so the MMAs of base tile t + 1 run while the
-// epilogue reads tile t.
-__global__ void __launch_bounds__(kTcThreads, 1) knn_tc_kernel(const __grid_constant__ CUtensorMap tq,
+__device__ __forceinline__ void tmem_ld(uint32_t (&v)[8], uint32_t taddr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld(uint32_t (&v)[16], uint32_t taddr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr));
+}
+
+// Wait for the warp's tensor-memory loads; the registers pass through, so that no use of
+// them can be moved above the wait.
+__device__ __forceinline__ void tmem_wait(uint32_t (&v)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait(uint32_t (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                 "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+               :
+               : "memory");
+}
+
+// A row's candidate list is a max-heap of `cand` keys (root = the worst kept key) and, per
+// epilogue warp that serves the row, a buffer of a few (score, id) pairs that were
+// below the root's score when they came; all with a stride of one slot per row.  Emptying
+// the buffer: the pairs that still beat the root replace it and sift down.  Returns the
+// root.  One copy of the code (the screening loop has to stay in the instruction cache).
+__device__ __noinline__ uint64_t heap_insert(uint64_t* heap, const uint2* pend, int cand, int waiting) {
+  uint64_t worst = heap[0];
+  for (int p = 0; p < waiting; ++p) {
+    const uint2 w = pend[(size_t)p * kRows];
+    const uint64_t key = ((uint64_t)ordered(__uint_as_float(w.x)) << 32) | w.y;
+    if (key >= worst) continue;
+    int i = 0;
+    for (;;) {
+      const int l = 2 * i + 1;
+      if (l >= cand) break;
+      const int r = l + 1;
+      const uint64_t hl = heap[(size_t)l * kRows];
+      const uint64_t hr = r < cand ? heap[(size_t)r * kRows] : 0ull;
+      const bool right = r < cand && hr > hl;
+      const uint64_t hc = right ? hr : hl;
+      if (hc <= key) break;
+      heap[(size_t)i * kRows] = hc;
+      i = right ? r : l;
+    }
+    heap[(size_t)i * kRows] = key;
+    worst = heap[0];
+  }
+  return worst;
+}
+
+// The two warps that serve the same 32 rows take turns at their heaps.  The holder never
+// waits for anything, so the lock is free again after one emptying; the attempts are
+// bounded all the same (false: gave up).
+__device__ __forceinline__ bool lock_rows(int* lock, int lane) {
+  int got = 0;
+  for (int i = 0; i < (1 << 22); ++i) {
+    if (lane == 0) got = atomicCAS(lock, 0, 1) == 0;
+    got = __shfl_sync(kFull, got, 0);
+    if (got) break;
+    __nanosleep(64);
+  }
+  __threadfence_block();
+  return got != 0;
+}
+__device__ __forceinline__ void unlock_rows(int* lock, int lane) {
+  __threadfence_block();
+  __syncwarp();
+  if (lane == 0) atomicExch(lock, 0);
+}
+
+struct RowList {
+  uint64_t* heap;
+  uint2* pend;
+  int* lock;            // null: one warp per row
+  volatile int* failed;  // set when a lock could not be had
+  int cand;
+  int waiting;
+  float worst_f;        // the root's score when this warp last saw it (never below the root's now)
+
+  // warp-wide
+  __device__ __forceinline__ void flush() {
+    const int lane = threadIdx.x & 31;
+    if (lock && !lock_rows(lock, lane)) {
+      *failed = 1;
+      waiting = 0;
+      return;
+    }
+    const uint64_t worst = heap_insert(heap, pend, cand, waiting);
+    waiting = 0;
+    worst_f = key_score(worst);
+    if (lock) unlock_rows(lock, lane);
+  }
+};
+
+// One group of scores of the row: a group whose best is not below any row's worst kept score
+// costs a fused multiply-add and a minimum per column.  A score equal to the worst kept one
+// may still enter by its id (the two halves' columns do not arrive in order): the keys decide.
+template <int kGroup, int kPend>
+__device__ __forceinline__ void screen(const uint32_t (&v)[kGroup], const float* xn, uint32_t id0, RowList& L) {
+  float sc[kGroup];
+#pragma unroll
+  for (int u = 0; u < kGroup; u += 4) {
+    const float4 x = *reinterpret_cast<const float4*>(xn + u);
+    sc[u] = __fmaf_rn(-2.0f, __uint_as_float(v[u]), x.x);  // +inf past the base
+    sc[u + 1] = __fmaf_rn(-2.0f, __uint_as_float(v[u + 1]), x.y);
+    sc[u + 2] = __fmaf_rn(-2.0f, __uint_as_float(v[u + 2]), x.z);
+    sc[u + 3] = __fmaf_rn(-2.0f, __uint_as_float(v[u + 3]), x.w);
+  }
+  float best = sc[0];
+#pragma unroll
+  for (int u = 1; u + 1 < kGroup; u += 2) best = fminf(best, fminf(sc[u], sc[u + 1]));
+  best = fminf(best, sc[kGroup - 1]);
+  if (!__any_sync(kFull, best <= L.worst_f)) return;
+  if (__any_sync(kFull, L.waiting > kPend - kGroup)) L.flush();
+#pragma unroll
+  for (int u = 0; u < kGroup; ++u) {
+    if (sc[u] <= L.worst_f) {
+      L.pend[(size_t)L.waiting * kRows] = make_uint2(__float_as_uint(sc[u]), id0 + (uint32_t)u);
+      ++L.waiting;
+    }
+  }
+}
+
+// Warp-specialised: EW epilogue warps read the accumulator (warp w the w % 4-th quarter of
+// the tensor-memory lanes, one query row per lane; with 8 warps each takes half of the
+// columns) and keep the candidates; the next warp issues the TMA loads; the last one the
+// MMAs into one of two accumulators (512 tensor-memory columns), so the MMAs of one tile run
+// while the epilogue reads the tile before.  ARES: the query tile's chunks are loaded once
+// per segment and stay in shared memory.
+//
+// What bounds it (1M x 128 rows, 10,000 queries, k = 10: 309k tiles, 0.57 us each at the
+// measured BF16 rate): the whole call takes 4.5 ms, 3.2 ms with nothing ever entering a list;
+// before, one tile at a time per SM behind one row of insertions, 9.2 ms.  Screening has to
+// stay in the instruction cache (all insertion code in one place: 13.3 -> 5.9 ms), two
+// epilogue warps per scheduler hide each other's tensor-memory loads (5.9 -> 5.3), and
+// without a barrier per tile they drift past each other's insertions (5.3 -> 4.5).  Equal
+// shares of the tiles replace whole query tiles x base slices, whose last wave was half
+// empty.  16 epilogue warps measured 4.7 ms, groups of 8 / 32 columns 5.4 / 4.6.
+template <bool PRECISE, bool ARES, int EW>
+__global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_constant__ CUtensorMap tq,
                                                                 const __grid_constant__ CUtensorMap tx, TcArgs a) {
+  constexpr int kEpi = EW * 32, kHalves = EW / 4, kTmaWarp = EW, kMmaWarp = EW + 1;
+  constexpr int kGroup = group_cols(EW), kPend = pend_slots(EW);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // 1024-byte alignment for the swizzled tiles
   unsigned char* sm = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-  const int S = a.stages;
-  unsigned char* sA = sm;                                  // S x 16 KB
-  unsigned char* sB = sA + S * kABytes;                    // S x 32 KB
+  const int S = a.stages, KC = a.kchunks;
+  const int na = ARES ? KC * (PRECISE ? 2 : 1) : S;        // query chunks in shared memory
+  unsigned char* sA = sm;                                  // na x 16 KB
+  unsigned char* sB = sA + na * kABytes;                   // S x 32 KB
   uint64_t* keys = reinterpret_cast<uint64_t*>(sB + S * kBBytes);  // [cand][128]
-  uint64_t* bars = keys + (size_t)a.cand * kEpiThreads;    // full[S], empty[S], acc_full[2], acc_empty[2]
+  uint2* pend = reinterpret_cast<uint2*>(keys + (size_t)a.cand * kRows);            // [kHalves][kPend][128]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(pend + (size_t)kHalves * kPend * kRows);  // full[S], empty[S], acc_full[2], acc_empty[2], a_full, a_empty
   uint64_t* full = bars;
   uint64_t* empty = bars + S;
   uint64_t* accf = bars + 2 * S;
   uint64_t* acce = accf + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
+  uint64_t* afull = acce + 2;
+  uint64_t* aempty = afull + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(aempty + 1);
   __shared__ volatile int s_fail;
-  __shared__ volatile int s_efail[2];  // the epilogue's own failure flag, by tile parity
-  __shared__ __align__(16) float s_xn[2][kTcN];  // ||x||^2 of the tile's base rows, double-buffered (read as float4)
+  __shared__ int s_lock[4];            // heaps of each quarter's rows
+  __shared__ __align__(16) float s_xn[EW][kTcN / kHalves];  // per epilogue warp: ||x||^2 of its columns' base rows
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long q0 = (long long)blockIdx.x * kTcM;
-  const int sl = blockIdx.y;
-  const long long r_begin = (long long)sl * a.slice;
-  const long long r_end = min(a.n, r_begin + a.slice);
-  const int ntiles = r_end > r_begin ? (int)((r_end - r_begin + kTcN - 1) / kTcN) : 0;
+  const long long u0 = a.share.start(blockIdx.x), u1 = a.share.start(blockIdx.x + 1);
+  const int bt = a.share.bt;
 
   if (tid == 0) {
     s_fail = 0;
-    s_efail[0] = s_efail[1] = 0;
+    for (int l = 0; l < 4; ++l) s_lock[l] = 0;
     for (int s = 0; s < S; ++s) {
       mbar_init(full + s, 1);
       mbar_init(empty + s, 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(accf + b, 1);
-      mbar_init(acce + b, kEpiThreads);
+      mbar_init(acce + b, EW);
     }
+    mbar_init(afull, 1);
+    mbar_init(aempty, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kMmaWarp) {
@@ -236,225 +445,339 @@ __global__ void __launch_bounds__(kTcThreads, 1) knn_tc_kernel(const __grid_cons
                  "r"(kAccCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  if (tid < kEpiThreads)
-    for (int i = 0; i < a.cand; ++i) keys[(size_t)i * kEpiThreads + tid] = kNoKey;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
+  // the steps of one 64-element chunk: which query part (hi 0, lo 1) meets which base part;
+  // with the query chunks resident a base chunk serves every query part it meets
+  constexpr int kSteps = PRECISE ? (ARES ? 2 : 3) : 1;
   if (warp == kTmaWarp) {
     if (lane == 0) {
-      uint32_t it = 0;
-      for (int t = 0; t < ntiles && !s_fail; ++t) {
-        const int r0 = (int)(r_begin + (long long)t * kTcN);
-        for (int kc = 0; kc < a.kchunks; ++kc, ++it) {
-          const int s = it % S;
-          const uint32_t use = it / S;
-          if (use > 0 && !mbar_wait(empty + s, (use - 1) & 1)) {
-            s_fail = 1;
+      uint32_t it = 0, seg = 0;
+      bool ok = true;
+      for (long long u = u0; u < u1 && ok; ++seg) {
+        const long long qt = u / bt, ue = min(u1, (qt + 1) * bt);
+        if (ARES) {
+          if (seg > 0 && !mbar_wait(aempty, (seg - 1) & 1)) {
+            ok = false;
             break;
           }
-          mbar_expect_tx(full + s, kABytes + kBBytes);
-          tma_load_2d(sA + s * kABytes, &tq, full + s, kc * kTcK, (int)q0);
-          tma_load_2d(sB + s * kBBytes, &tx, full + s, kc * kTcK, r0);
+          mbar_expect_tx(afull, (uint32_t)(na * kABytes));
+          for (int c = 0; c < na; ++c) tma_load_2d(sA + c * kABytes, &tq, afull, c * kTcK, (int)(qt * kTcM));
         }
+        for (; u < ue && ok; ++u) {
+          if (s_fail) {
+            ok = false;
+            break;
+          }
+          const int r0 = (int)((u - qt * bt) * kTcN);
+          for (int kc = 0; kc < KC && ok; ++kc) {
+#pragma unroll
+            for (int st = 0; st < kSteps; ++st, ++it) {
+              const int s = it % S;
+              const uint32_t use = it / S;
+              if (use > 0 && !mbar_wait(empty + s, (use - 1) & 1)) {
+                ok = false;
+                break;
+              }
+              const int xpart = PRECISE ? (ARES ? st : st == 2) : 0;
+              const int qpart = PRECISE && !ARES && st == 1;
+              mbar_expect_tx(full + s, ARES ? kBBytes : kABytes + kBBytes);
+              if (!ARES) tma_load_2d(sA + s * kABytes, &tq, full + s, (qpart * KC + kc) * kTcK, (int)(qt * kTcM));
+              tma_load_2d(sB + s * kBBytes, &tx, full + s, (xpart * KC + kc) * kTcK, r0);
+            }
+          }
+        }
+        u = ue;
       }
+      if (!ok) s_fail = 1;
     }
   } else if (warp == kMmaWarp) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16(kTcM, kTcN);
-      uint32_t it = 0;
-      for (int t = 0; t < ntiles && !s_fail; ++t) {
-        const int b = t & 1;
-        const uint32_t ub = (uint32_t)t >> 1;
-        if (ub > 0 && !mbar_wait(acce + b, (ub - 1) & 1)) {  // the epilogue is done with this accumulator
-          s_fail = 1;
+      uint32_t it = 0, seg = 0, t = 0;
+      bool ok = true;
+      for (long long u = u0; u < u1 && ok; ++seg) {
+        const long long qt = u / bt, ue = min(u1, (qt + 1) * bt);
+        if (ARES && !mbar_wait(afull, seg & 1)) {
+          ok = false;
           break;
         }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t dacc = tmem + (uint32_t)(b * kTcN);
-        bool ok = true;
-        for (int kc = 0; kc < a.kchunks; ++kc, ++it) {
-          const int s = it % S;
-          const uint32_t use = it / S;
-          if (!mbar_wait(full + s, use & 1)) {
+        for (; u < ue && ok; ++u, ++t) {
+          const uint32_t b = t & 1, ub = t >> 1;
+          if (s_fail || (ub > 0 && !mbar_wait(acce + b, (ub - 1) & 1))) {  // the epilogue is done with this accumulator
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t dacc = tmem + b * kTcN;
+          uint32_t acc = 0;  // the tile's first MMA overwrites the accumulator
+          auto mma = [&](const unsigned char* pa, const unsigned char* pb) {
 #pragma unroll
-          for (int k16 = 0; k16 < kTcK / 16; ++k16) {
-            const uint64_t da = smem_desc_sw128(sA + s * kABytes + k16 * 32);
-            const uint64_t db = smem_desc_sw128(sB + s * kBBytes + k16 * 32);
-            const uint32_t acc = (kc > 0 || k16 > 0) ? 1u : 0u;
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t"
-                "setp.ne.b32 p, %4, 0;\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dacc),
-                "l"(da), "l"(db), "r"(idesc), "r"(acc));
+            for (int k16 = 0; k16 < kTcK / 16; ++k16) {
+              const uint64_t da = smem_desc_sw128(pa + k16 * 32);
+              const uint64_t db = smem_desc_sw128(pb + k16 * 32);
+              asm volatile(
+                  "{\n\t.reg .pred p;\n\t"
+                  "setp.ne.b32 p, %4, 0;\n\t"
+                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dacc),
+                  "l"(da), "l"(db), "r"(idesc), "r"(acc));
+              acc = 1;
+            }
+          };
+          for (int kc = 0; kc < KC && ok; ++kc) {
+#pragma unroll
+            for (int st = 0; st < kSteps; ++st, ++it) {
+              const int s = it % S;
+              if (!mbar_wait(full + s, (it / S) & 1)) {
+                ok = false;
+                break;
+              }
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              if (ARES) {
+                mma(sA + kc * kABytes, sB + s * kBBytes);
+                if (PRECISE && st == 0) mma(sA + (KC + kc) * kABytes, sB + s * kBBytes);
+              } else {
+                mma(sA + s * kABytes, sB + s * kBBytes);
+              }
+              asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                               smem_u32(empty + s))
+                           : "memory");
+            }
           }
+          if (!ok) break;
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_u32(empty + s))
+                           smem_u32(accf + b))
                        : "memory");
         }
-        if (!ok) {
-          s_fail = 1;
-          break;
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         smem_u32(accf + b))
-                     : "memory");
+        if (ARES && ok && ue < u1)  // the segment's MMAs are done with the query chunks
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                           smem_u32(aempty))
+                       : "memory");
+        u = ue;
       }
+      if (!ok) s_fail = 1;
     }
   } else {
-    // epilogue: thread tid owns accumulator row tid (query q0 + tid); a score is compared
-    // with the list's worst as a float first and becomes a key only when it may enter
-    uint64_t* mine = keys + tid;
-    for (int t = 0; t < ntiles; ++t) {
-      const int b = t & 1;
-      const long long r0 = r_begin + (long long)t * kTcN;
-      for (int j = tid; j < kTcN; j += kEpiThreads) s_xn[b][j] = (r0 + j < r_end) ? __ldg(a.xnorm + r0 + j) : INFINITY;
-      // a failed wait is flagged in this tile's slot before the barrier and read after it,
-      // so all four warps leave together (a thread one tile ahead writes the other slot)
-      if (!mbar_wait(accf + b, ((uint32_t)t >> 1) & 1)) {
-        s_efail[b] = 1;
-        s_fail = 1;
-      }
-      epilogue_sync();
-      if (s_efail[b]) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      uint64_t worst = mine[0];  // the root of the row's max-heap of kept keys
-      float worst_f = key_score(worst);
-      for (int c0 = 0; c0 < kTcN; c0 += 32) {
-        uint32_t v[32];
-        __syncwarp();  // tcgen05.ld is warp-collective
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * kTcN + c0);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-            "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-            "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-              "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
-              "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
-              "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        // screen 32 scores against the list's worst score: a bit per column that may enter.
-        // Columns arrive in increasing order, so a score equal to the worst one has a larger
-        // key than every kept key with that score and never enters: the test is strict.
-        float sc[32];
-        uint32_t mask = 0;
-        const float4* xn4 = reinterpret_cast<const float4*>(&s_xn[b][c0]);
+    // epilogue: a lane owns accumulator row `row` (query qt * 128 + row), shared with the
+    // warp of the other half
+    const int quarter = warp & 3, half = warp >> 2, row = quarter * 32 + lane;
+    constexpr int kCols = kTcN / kHalves;
+    RowList list{keys + row, pend + (size_t)half * kPend * kRows + row, kHalves > 1 ? &s_lock[quarter] : nullptr,
+                 &s_fail, a.cand, 0, FLT_MAX};
+    uint32_t t = 0;
+    bool ok = true;
+    // ||x||^2 of the warp's columns of the next tile, loaded a tile ahead
+    constexpr int kNorms = kCols / 32;
+    float xn[kNorms];
+    float* my_xn = s_xn[warp];
+    auto load_norms = [&](int tile) {  // tile of the base
+      const long long r = (long long)tile * kTcN + half * kCols + lane;
 #pragma unroll
-        for (int j4 = 0; j4 < 8; ++j4) {
-          const float4 xn = xn4[j4];
-          sc[4 * j4 + 0] = __fmaf_rn(-2.0f, __uint_as_float(v[4 * j4 + 0]), xn.x);  // +inf past the slice
-          sc[4 * j4 + 1] = __fmaf_rn(-2.0f, __uint_as_float(v[4 * j4 + 1]), xn.y);
-          sc[4 * j4 + 2] = __fmaf_rn(-2.0f, __uint_as_float(v[4 * j4 + 2]), xn.z);
-          sc[4 * j4 + 3] = __fmaf_rn(-2.0f, __uint_as_float(v[4 * j4 + 3]), xn.w);
+      for (int j = 0; j < kNorms; ++j) xn[j] = r + 32 * j < a.n ? __ldg(a.xnorm + r + 32 * j) : INFINITY;
+    };
+    if (u0 < u1) load_norms((int)(u0 % bt));
+    for (long long u = u0; u < u1;) {
+      const long long qt = u / bt, ue = min(u1, (qt + 1) * bt);
+      for (int i = half; i < a.cand; i += kHalves) list.heap[(size_t)i * kRows] = kNoKey;
+      list.worst_f = FLT_MAX;
+      quarter_sync<EW>(quarter);
+      // after a failed wait the warp only keeps up with its barriers
+      for (; u < ue && ok; ++u, ++t) {
+        const uint32_t b = t & 1;
+        const uint32_t id0 = a.row0 + (uint32_t)((u - qt * bt) * kTcN) + half * kCols;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) mask |= (sc[4 * j4 + u] < worst_f ? 1u : 0u) << (4 * j4 + u);
+        for (int j = 0; j < kNorms; ++j) my_xn[lane + 32 * j] = xn[j];
+        if (u + 1 < u1) load_norms(u + 1 < ue ? (int)(u + 1 - qt * bt) : 0);
+        if (!mbar_wait(accf + b, (t >> 1) & 1)) s_fail = 1;
+        __syncwarp();
+        ok = !__any_sync(kFull, s_fail != 0);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + b * kTcN + half * kCols;
+        // two loads in flight: one is screened while the next arrives
+        uint32_t va[kGroup], vb[kGroup];
+        tmem_ld(va, taddr);  // warp-collective
+        tmem_wait(va);
+#pragma unroll 1
+        for (int c0 = 0; c0 < kCols; c0 += 2 * kGroup) {
+          tmem_ld(vb, taddr + c0 + kGroup);
+          screen<kGroup, kPend>(va, my_xn + c0, id0 + c0, list);
+          __syncwarp();
+          tmem_wait(vb);
+          if (c0 + 2 * kGroup < kCols) tmem_ld(va, taddr + c0 + 2 * kGroup);
+          screen<kGroup, kPend>(vb, my_xn + c0 + kGroup, id0 + c0 + kGroup, list);
+          __syncwarp();
+          tmem_wait(va);
         }
-        // one set bit per lane per iteration, so lanes insert side by side (a single copy
-        // of the insertion code; the score is picked out of the registers by selects)
-        while (mask) {
-          const int j = __ffs(mask) - 1;
-          mask &= mask - 1;
-          float sj = sc[0];
-#pragma unroll
-          for (int u = 1; u < 32; ++u) sj = (j == u) ? sc[u] : sj;
-          const long long col = r0 + c0 + j;
-          const uint64_t key = ((uint64_t)ordered(sj) << 32) | (uint32_t)col;
-          if (col < r_end && key < worst) {
-            // replace the heap's root (the worst kept key) and sift down
-            int i = 0;
-            for (;;) {
-              const int l = 2 * i + 1;
-              if (l >= a.cand) break;
-              const int r = l + 1;
-              const uint64_t hl = mine[(size_t)l * kEpiThreads];
-              const uint64_t hr = r < a.cand ? mine[(size_t)r * kEpiThreads] : 0ull;
-              const int c = (r < a.cand && hr > hl) ? r : l;
-              const uint64_t hc = c == r ? hr : hl;
-              if (hc <= key) break;
-              mine[(size_t)i * kEpiThreads] = hc;
-              i = c;
-            }
-            mine[(size_t)i * kEpiThreads] = key;
-            worst = mine[0];
-            worst_f = key_score(worst);
-          }
-        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce + b);  // this warp is done with the accumulator
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(acce + b);  // this thread is done with the accumulator
+      u = ue;
+      list.flush();
+      quarter_sync<EW>(quarter);
+      if (ok && qt * kTcM + row < a.nq) {
+        const int seg = a.seg0 + blockIdx.x - a.share.cta_of(qt * bt);
+        uint64_t* o = a.out + ((size_t)(qt * kTcM + row) * a.nseg + seg) * a.cand;
+        for (int i = half; i < a.cand; i += kHalves) o[i] = list.heap[(size_t)i * kRows];
+      }
+      quarter_sync<EW>(quarter);  // the lists are written before they are emptied for the next query tile
     }
   }
   __syncthreads();
-  if (s_fail) {
-    if (tid == 0) atomicExch(a.err, 1);
-  } else if (tid < kEpiThreads && q0 + tid < a.nq) {
-    uint64_t* o = a.out + ((size_t)(q0 + tid) * a.nslice + sl) * a.cand;
-    for (int i = 0; i < a.cand; ++i) o[i] = keys[(size_t)i * kEpiThreads + tid];
-  }
+  if (s_fail && tid == 0) atomicExch(a.err, 1);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == kMmaWarp)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAccCols));
 }
 
-// Exact FP32 distances of every query's candidates (one warp per query, one candidate per
-// lane at a time, a sequential sum over the dimensions), then the k smallest by (dist, id).
-constexpr int kFinWarps = 4;
-__global__ void __launch_bounds__(kFinWarps * 32) knn_tc_finalize(const float* __restrict__ X, const float* __restrict__ Q,
-                                                                  long long nq, int d, const uint64_t* __restrict__ cand,
-                                                                  int ncand, int P, int k, int32_t* __restrict__ ids_out,
-                                                                  float* __restrict__ dists_out) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint64_t* s_key = reinterpret_cast<uint64_t*>(smem_raw) + (size_t)warp * P;
-  for (long long q = (long long)blockIdx.x * kFinWarps + warp; q < nq; q += (long long)gridDim.x * kFinWarps) {
-    const float* qv = Q + (size_t)q * d;
-    for (int i = lane; i < P; i += 32) {
-      uint64_t key = kNoKey;
-      if (i < ncand) {
-        const uint64_t c = cand[(size_t)q * ncand + i];
-        if (c != kNoKey) {
-          const uint32_t id = (uint32_t)(c & 0xffffffffu);
-          const float* xv = X + (size_t)id * d;
-          float acc = 0.0f;
-          for (int t = 0; t < d; ++t) {
-            const float df = __ldg(qv + t) - __ldg(xv + t);
-            acc = acc + df * df;
-          }
-          key = pack_key(acc, (int32_t)id);
+struct FinArgs {
+  const float* X;
+  const float* Q;
+  long long nq;
+  int d;
+  const uint64_t* cand;  // [nq][nseg][cand]
+  int nseg, ncand1;      // segments, candidates per segment
+  int P;                 // power of two >= nseg * ncand1
+  int k;
+  int32_t* ids_out;
+  float* dists_out;
+  const unsigned* xmax;  // bits of the largest ||x||^2
+  float c_dot;           // |score error| <= c_dot ||q|| ||x||max + c_norm ||x||max^2
+  float c_norm;
+  // precise form: queries whose result is not proven
+  const int* err;
+  int* left_count;
+  int32_t* left;
+};
+
+// One group of WPQ warps per query.
+template <int WPQ>
+__device__ __forceinline__ void group_sync() {
+  if (WPQ == 1) __syncwarp();
+  else __syncthreads();
+}
+
+template <int WPQ>
+__device__ __forceinline__ void group_sort(uint64_t* key, int P, int t) {
+  for (int size = 2; size <= P; size <<= 1) {
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      for (int i = t; i < (P >> 1); i += WPQ * 32) {
+        const int lo = 2 * i - (i & (stride - 1));
+        const int hi = lo + stride;
+        const uint64_t x = key[lo], y = key[hi];
+        if ((x > y) == ((lo & size) == 0)) {
+          key[lo] = y;
+          key[hi] = x;
         }
+      }
+      group_sync<WPQ>();
+    }
+  }
+}
+
+constexpr int kFinWarps = 4;      // warps per CTA where a warp takes a query
+constexpr int kFinGroupWarps = 8;  // where a CTA takes one
+template <int WPQ, bool PRECISE>
+__global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_finalize(FinArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int kQueries = WPQ == 1 ? kFinWarps : 1;  // per CTA
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = WPQ == 1 ? lane : threadIdx.x;
+  uint64_t* s_key = reinterpret_cast<uint64_t*>(smem_raw) + (size_t)(WPQ == 1 ? warp : 0) * a.P;
+  const int d = a.d, d4 = d >> 2, ncand = a.nseg * a.ncand1;
+  const double xm2 = (double)__uint_as_float(*a.xmax), xm = sqrt(xm2);
+  for (long long q = (long long)blockIdx.x * kQueries + (WPQ == 1 ? warp : 0); q < a.nq; q += (long long)gridDim.x * kQueries) {
+    const float4* qv = reinterpret_cast<const float4*>(a.Q + (size_t)q * d);
+    // ||q||^2, the same in every warp
+    double q2 = 0.0;
+    for (int c = lane; c < d4; c += 32) {
+      const float4 v = __ldg(qv + c);
+      q2 += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q2 += __shfl_xor_sync(kFull, q2, o);
+    const double err = (double)a.c_dot * sqrt(q2) * xm + (double)a.c_norm * xm2;
+    const uint64_t* src = a.cand + (size_t)q * ncand;
+    for (int i = t; i < a.P; i += WPQ * 32) s_key[i] = i < ncand ? src[i] : kNoKey;
+    // the smallest root of a full list: no row left out scored below it
+    uint64_t left_out = kNoKey;
+    if (PRECISE) {
+      for (int i = lane; i < a.nseg; i += 32) left_out = min(left_out, src[(size_t)i * a.ncand1]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) left_out = min(left_out, (uint64_t)__shfl_xor_sync(kFull, (unsigned long long)left_out, o));
+    }
+    group_sync<WPQ>();
+    group_sort<WPQ>(s_key, a.P, t);
+    // a candidate more than two error bounds above the k-th score is farther than k others,
+    // also in FP32
+    const double fp = (double)(d + 4) * 0x1p-23;
+    const uint64_t kth = s_key[a.k - 1];
+    const double thr = kth == kNoKey ? INFINITY : (double)key_score(kth) + 2.0 * err + fp * fabs((double)key_score(kth) + err + q2);
+    int m = 0;  // candidates to measure: the first m
+    {
+      int lo = 0, hi = a.P;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const uint64_t key = s_key[mid];
+        if (key != kNoKey && !((double)key_score(key) > thr)) lo = mid + 1; else hi = mid;
+      }
+      m = lo;
+    }
+    int P2 = 1;
+    while (P2 < m) P2 <<= 1;
+    if (P2 < a.k) {
+      while (P2 < a.k) P2 <<= 1;
+      P2 = min(P2, a.P);
+    }
+    group_sync<WPQ>();
+    for (int i = t; i < P2; i += WPQ * 32) {
+      uint64_t key = kNoKey;
+      if (i < m) {
+        const uint32_t id = (uint32_t)(s_key[i] & 0xffffffffu);
+        const float4* xv = reinterpret_cast<const float4*>(a.X + (size_t)id * d);
+        float acc = 0.0f;
+#pragma unroll 4
+        for (int c = 0; c < d4; ++c) {
+          const float4 x = __ldg(xv + c), y = __ldg(qv + c);
+          const float e0 = y.x - x.x, e1 = y.y - x.y, e2 = y.z - x.z, e3 = y.w - x.w;
+          if (PRECISE) {  // the FFMA kernel's sum
+            acc = fmaf(e0, e0, acc);
+            acc = fmaf(e1, e1, acc);
+            acc = fmaf(e2, e2, acc);
+            acc = fmaf(e3, e3, acc);
+          } else {
+            acc = acc + e0 * e0;
+            acc = acc + e1 * e1;
+            acc = acc + e2 * e2;
+            acc = acc + e3 * e3;
+          }
+        }
+        key = pack_key(acc, (int32_t)id);
       }
       s_key[i] = key;
     }
-    __syncwarp();
-    for (int size = 2; size <= P; size <<= 1) {
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        for (int i = lane; i < (P >> 1); i += 32) {
-          const int lo = 2 * i - (i & (stride - 1));
-          const int hi = lo + stride;
-          const uint64_t x = s_key[lo], y = s_key[hi];
-          if ((x > y) == ((lo & size) == 0)) {
-            s_key[lo] = y;
-            s_key[hi] = x;
-          }
-        }
-        __syncwarp();
+    group_sync<WPQ>();
+    group_sort<WPQ>(s_key, P2, t);
+    for (int j = t; j < a.k; j += WPQ * 32) {
+      const uint64_t key = j < P2 ? s_key[j] : kNoKey;
+      a.ids_out[(size_t)q * a.k + j] = key == kNoKey ? -1 : key_id(key);
+      a.dists_out[(size_t)q * a.k + j] = key == kNoKey ? INFINITY : key_dist(key);
+    }
+    if (PRECISE && t == 0) {
+      bool proven = *a.err == 0 && isfinite(xm2) && isfinite(q2) && xm2 >= 1e-24 && (q2 >= 1e-24 || q2 == 0.0);
+      if (left_out != kNoKey) {
+        const uint64_t last = s_key[a.k - 1];
+        proven = proven && last != kNoKey &&
+                 ((double)key_score(left_out) - err + q2) * (1.0 - fp) > (double)key_dist(last) * (1.0 + 0x1p-20);
       }
+      if (!proven) a.left[atomicAdd(a.left_count, 1)] = (int32_t)q;
     }
-    for (int j = lane; j < k; j += 32) {
-      const uint64_t key = s_key[j];
-      ids_out[(size_t)q * k + j] = key == kNoKey ? -1 : key_id(key);
-      dists_out[(size_t)q * k + j] = key == kNoKey ? INFINITY : key_dist(key);
-    }
-    __syncwarp();
+    group_sync<WPQ>();
   }
 }
 
@@ -490,46 +813,203 @@ bool make_map(CUtensorMap* m, const void* base, long long rows, int pitch, int b
 
 }  // namespace
 
-int knn_tc_pitch(int d) { return (d + kTcK - 1) / kTcK * kTcK; }
+namespace {
 
-int knn_tc_cand(int k) { return k + 16; }
+constexpr size_t kTcPad = 256;
+size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+int tc_pitch(int d) { return (d + kTcK - 1) / kTcK * kTcK; }
 
-int knn_tc_slices(long long n, long long nq, int k, int sms) {
-  // One CTA per SM; a CTA pays for its base tiles and for the insertions into its rows'
-  // candidate heaps, about cand (1 + ln(rows / cand)) per row and slice (a random stream),
-  // worth ~64 tiles of MMA and screening per unit of that log term (measured on GB300 at
-  // d = 128 and 960).  Pick the slice count s minimising waves(s) x per-CTA cost, among
-  // slices of >= 4 tiles and at most kMaxCandTotal candidates per query.
+// The plan of one call: how the tiles are shared and what the scratch holds.
+struct TcPlan {
+  int pitch, cand, nseg, slabs;
+  long long slab_rows;  // base rows converted at a time
+  TcShare share;        // of a full slab
+  size_t xb, qb, xnorm, cand_buf, flags, total;  // scratch offsets
+};
+
+TcShare tc_share(long long n, long long nq, int cand, int slabs, int sms) {
+  TcShare s;
   const long long qt = (nq + kTcM - 1) / kTcM;
-  const int cand = knn_tc_cand(k);
-  long long max_s = (n + 4LL * kTcN - 1) / (4LL * kTcN);
-  const long long max_c = kMaxCandTotal / cand;
-  if (max_s > max_c) max_s = max_c;
-  if (max_s < 1) max_s = 1;
-  long long best = 1;
-  double best_cost = -1.0;
-  for (long long s = 1; s <= max_s; ++s) {
-    const long long waves = (qt * s + sms - 1) / sms;
-    const double rows = (double)((n + s - 1) / s);
-    const double tiles = ceil(rows / kTcN);
-    const double ins = rows > cand ? 1.0 + log(rows / cand) : 1.0;
-    const double cost = (double)waves * (tiles + 64.0 * ins);
-    if (best_cost < 0.0 || cost < best_cost) {
-      best_cost = cost;
-      best = s;
-    }
-  }
-  return (int)best;
+  s.bt = (int)((n + kTcN - 1) / kTcN);
+  s.units = qt * s.bt;
+  // one CTA per SM; no more than kMaxCandTotal candidates per query over its segments (a
+  // query tile's share spans at most ceil(G / qt) + 1 CTAs), and segments of at least 4
+  // tiles, below which the lists' start-up would outweigh the tiles
+  long long G = sms;
+  const long long most = kMaxCandTotal / ((long long)cand * slabs);
+  if (most >= 2) G = std::min(G, std::max(1LL, (most - 1) * qt));
+  else G = std::min(G, qt);
+  G = std::min(G, std::max(1LL, s.units / 4));
+  s.G = (int)std::max(1LL, G);
+  return s;
 }
+
+// The longest list whose launch fits in shared memory (4 epilogue warps, two stages of query
+// and base chunks).  The precise form serves k up to 8 below it: its lists hold 16 more than
+// k, fewer where shared memory ends (a shorter slack only proves fewer queries).
+constexpr int kMaxCand = 113;
+
+// precise: the base is converted in slabs of at most 1 GiB.  False: not served.
+bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcPlan* p) {
+  p->pitch = tc_pitch(d);
+  p->cand = precise ? std::min(k + 16, kMaxCand) : k + 16;
+  if (p->cand < k + 8 || p->cand > kMaxCand) return false;
+  const size_t row = (size_t)p->pitch * 2 * (precise ? 2 : 1);
+  p->slab_rows = n;
+  p->slabs = 1;
+  if (precise) {
+    const long long fit = std::max<long long>(kTcN, (long long)(((size_t)1 << 30) / row) / kTcN * kTcN);
+    p->slabs = (int)((n + fit - 1) / fit);
+    p->slab_rows = p->slabs > 1 ? fit : n;
+  }
+  p->share = tc_share(p->slab_rows, nq, p->cand, p->slabs, sms);
+  int seg = p->share.max_segments();
+  if (p->slabs > 1) {
+    const TcShare last = tc_share(n - (long long)(p->slabs - 1) * p->slab_rows, nq, p->cand, p->slabs, sms);
+    seg = std::max(seg, last.max_segments());
+  }
+  p->nseg = seg * p->slabs;
+  if ((long long)p->nseg * p->cand > kMaxCandTotal && p->nseg > 1) return false;
+  size_t o = 0;
+  p->xb = o;
+  o += up256((size_t)p->slab_rows * row);
+  p->qb = o;
+  o += up256((size_t)nq * row);
+  p->xnorm = o;
+  o += up256((size_t)p->slab_rows * 4);
+  p->cand_buf = o;
+  o += up256((size_t)nq * p->nseg * p->cand * 8);
+  p->flags = o;  // xmax, err, left count
+  o += kTcPad;
+  p->total = o;
+  return true;
+}
+
+template <bool PRECISE, bool ARES, int EW>
+cudaError_t launch_tc(const CUtensorMap& mq, const CUtensorMap& mx, TcArgs ta, int maxsm, cudaStream_t st, bool* fits) {
+  auto fn = knn_tc_kernel<PRECISE, ARES, EW>;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+  if (e != cudaSuccess) return e;
+  const size_t room = (size_t)maxsm - fa.sharedSizeBytes;  // the kernel's static shared memory comes off the top
+  // as many ring stages as fit beside the lists and the resident query chunks (one CTA per SM
+  // either way: the two accumulators take all 512 tensor-memory columns)
+  const size_t fixed = 1024 + (size_t)(ta.cand + EW / 4 * pend_slots(EW)) * kRows * 8 + (2 * kMaxStages + 6) * 8 + 16 +
+                       (ARES ? (size_t)ta.kchunks * (PRECISE ? 2 : 1) * kABytes : 0);
+  const size_t stage = kBBytes + (ARES ? 0 : kABytes);
+  int stages = kMaxStages;
+  const int least = ARES ? 3 : 2;
+  while (stages > least && fixed + (size_t)stages * stage > room) --stages;
+  size_t smem = fixed + (size_t)stages * stage;
+  *fits = smem <= room;
+  if (!*fits) return cudaSuccess;
+  const size_t one_per_sm = ((size_t)maxsm) / 2 + 1024;  // never two CTAs on one SM
+  if (smem < one_per_sm) smem = one_per_sm;
+  ta.stages = stages;
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  fn<<<(unsigned)ta.share.G, (EW + 2) * 32, smem, st>>>(mq, mx, ta);
+  return cudaGetLastError();
+}
+
+// The candidate lists and their evaluation; `left` / `left_count` (precise): the queries
+// whose result is not proven.
+template <bool PRECISE>
+cudaError_t run_tc(const TcPlan& p, const float* X, long long n, int d, const float* Q, long long nq, int k,
+                   int32_t* ids_out, float* dists_out, unsigned char* w, int* err, int* left_count, int32_t* left,
+                   int sms, cudaStream_t st) {
+  int dev = 0, maxsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  __nv_bfloat16* xb = reinterpret_cast<__nv_bfloat16*>(w + p.xb);
+  __nv_bfloat16* qb = reinterpret_cast<__nv_bfloat16*>(w + p.qb);
+  float* xnorm = reinterpret_cast<float*>(w + p.xnorm);
+  uint64_t* cand_buf = reinterpret_cast<uint64_t*>(w + p.cand_buf);
+  unsigned* xmax = reinterpret_cast<unsigned*>(w + p.flags);
+  cudaError_t e = cudaMemsetAsync(cand_buf, 0xff, (size_t)nq * p.nseg * p.cand * 8, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(xmax, 0, sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  const int cols = p.pitch * (PRECISE ? 2 : 1);
+  const int cg = sms * 8;
+  convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (nq + 7) / 8), 256, 0, st>>>(Q, nq, d, p.pitch, qb,
+                                                                                               nullptr, nullptr);
+  CUtensorMap mq;
+  if (!make_map(&mq, qb, nq, cols, kTcM)) return cudaErrorNotSupported;
+  for (int s = 0; s < p.slabs; ++s) {
+    const long long r0 = (long long)s * p.slab_rows, rows = std::min(p.slab_rows, n - r0);
+    convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (rows + 7) / 8), 256, 0, st>>>(
+        X + (size_t)r0 * d, rows, d, p.pitch, xb, xnorm, xmax);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    CUtensorMap mx;
+    if (!make_map(&mx, xb, rows, cols, kTcN)) return cudaErrorNotSupported;
+    TcArgs ta;
+    ta.xnorm = xnorm;
+    ta.n = rows;
+    ta.nq = nq;
+    ta.share = rows == p.slab_rows ? p.share : tc_share(rows, nq, p.cand, p.slabs, sms);
+    ta.kchunks = p.pitch / kTcK;
+    ta.cand = p.cand;
+    ta.row0 = (uint32_t)r0;
+    ta.nseg = p.nseg;
+    ta.seg0 = s * (p.nseg / p.slabs);
+    ta.out = cand_buf;
+    ta.err = err;
+    bool fits = false;
+    e = launch_tc<PRECISE, true, 8>(mq, mx, ta, maxsm, st, &fits);
+    if (e == cudaSuccess && !fits) e = launch_tc<PRECISE, false, 8>(mq, mx, ta, maxsm, st, &fits);
+    if (e == cudaSuccess && !fits) e = launch_tc<PRECISE, false, 4>(mq, mx, ta, maxsm, st, &fits);
+    if (e == cudaSuccess && !fits) e = cudaErrorInvalidConfiguration;
+    if (e != cudaSuccess) return e;
+  }
+  FinArgs fa{};
+  fa.X = X;
+  fa.Q = Q;
+  fa.nq = nq;
+  fa.d = d;
+  fa.cand = cand_buf;
+  fa.nseg = p.nseg;
+  fa.ncand1 = p.cand;
+  fa.P = 1;
+  while (fa.P < p.nseg * p.cand || fa.P < k) fa.P <<= 1;
+  fa.k = k;
+  fa.ids_out = ids_out;
+  fa.dists_out = dists_out;
+  fa.xmax = xmax;
+  // Score error, relative to ||q|| ||x||: the terms dropped or rounded (BF16's unit roundoff
+  // is 2^-8: 2 (2^-8 + 2^-18) alone, 3.05 2^-16 for the two-term sums), and the FP32
+  // accumulation, at most 2^-23 per product (each step of 16 aligns its products and the
+  // accumulator to the largest and truncates); times 2 for -2 q.x, plus the last rounding.
+  const double products = (double)p.pitch * (PRECISE ? 3 : 1);
+  fa.c_dot = (float)(2.0 * ((PRECISE ? 3.05 * 0x1p-16 : 2.02 * 0x1p-8) + products * 0x1p-23) + 0x1p-21);
+  fa.c_norm = (float)((d / 32 + 10) * 0x1p-23);
+  fa.err = err;
+  fa.left_count = left_count;
+  fa.left = left;
+  // a warp per query, or a CTA per query where the lists are long or the queries few
+  if (fa.P <= 1024 && nq >= 2LL * sms) {
+    const size_t sm = (size_t)fa.P * 8 * kFinWarps;
+    e = cudaFuncSetAttribute(knn_tc_finalize<1, PRECISE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    const long long g = std::min<long long>((nq + kFinWarps - 1) / kFinWarps, (long long)sms * 16);
+    knn_tc_finalize<1, PRECISE><<<(unsigned)g, kFinWarps * 32, sm, st>>>(fa);
+  } else {
+    const size_t sm = (size_t)fa.P * 8;
+    e = cudaFuncSetAttribute(knn_tc_finalize<kFinGroupWarps, PRECISE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    const long long g = std::min<long long>(nq, (long long)sms * 8);
+    knn_tc_finalize<kFinGroupWarps, PRECISE><<<(unsigned)g, kFinGroupWarps * 32, sm, st>>>(fa);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace
 
 int knn_tc_max_k() { return kMaxK; }
 
 size_t knn_tc_scratch_bytes(long long n, long long nq, int d, int k, int sms) {
-  const size_t pitch = (size_t)knn_tc_pitch(d);
-  const size_t ns = (size_t)knn_tc_slices(n, nq, k, sms);
-  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  return up((size_t)n * pitch * 2) + up((size_t)nq * pitch * 2) + up((size_t)n * 4) +
-         up((size_t)nq * ns * knn_tc_cand(k) * 8) + 256;
+  TcPlan p;
+  return tc_plan(n, nq, d, k, false, sms, &p) ? p.total : 0;
 }
 
 cudaError_t launch_knn_tc(const float* X, long long n, int d, const float* Q, long long nq, int k, int32_t* ids_out,
@@ -538,72 +1018,32 @@ cudaError_t launch_knn_tc(const float* X, long long n, int d, const float* Q, lo
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int pitch = knn_tc_pitch(d);
-  const int ns = knn_tc_slices(n, nq, k, sms);
-  const int cand = knn_tc_cand(k);
-  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  TcPlan p;
+  if (!tc_plan(n, nq, d, k, false, sms, &p)) return cudaErrorInvalidConfiguration;
+  return run_tc<false>(p, X, n, d, Q, nq, k, ids_out, dists_out, static_cast<unsigned char*>(scratch), err_flag, nullptr,
+                       nullptr, sms, st);
+}
+
+// ---- exact brute force: the precise form, and the FFMA kernel for what it leaves -----------
+
+size_t knn_exact_scratch_bytes(long long n, long long nq, int d, int k, int sms) {
+  TcPlan p;
+  return tc_plan(n, nq, d, k, true, sms, &p) ? p.total + up256((size_t)nq * 4) : 0;
+}
+
+cudaError_t launch_knn_exact(const float* X, long long n, int d, const float* Q, long long nq, int k, int32_t* ids_out,
+                             float* dists_out, void* scratch, void* ffma_scratch, int sms, cudaStream_t st) {
+  TcPlan p;
+  if (!tc_plan(n, nq, d, k, true, sms, &p)) return cudaErrorInvalidConfiguration;
   unsigned char* w = static_cast<unsigned char*>(scratch);
-  __nv_bfloat16* xb = reinterpret_cast<__nv_bfloat16*>(w);
-  w += up((size_t)n * pitch * 2);
-  __nv_bfloat16* qb = reinterpret_cast<__nv_bfloat16*>(w);
-  w += up((size_t)nq * pitch * 2);
-  float* xnorm = reinterpret_cast<float*>(w);
-  w += up((size_t)n * 4);
-  uint64_t* cand_buf = reinterpret_cast<uint64_t*>(w);
-  (void)err_flag;
-
-  const int cg = sms * 8;
-  convert_bf16_kernel<<<cg, 256, 0, st>>>(X, n, d, pitch, xb, xnorm);
-  convert_bf16_kernel<<<cg, 256, 0, st>>>(Q, nq, d, pitch, qb, nullptr);
-  cudaError_t e = cudaGetLastError();
+  int* err = reinterpret_cast<int*>(w + p.flags) + 1;
+  int* left_count = err + 1;
+  int32_t* left = reinterpret_cast<int32_t*>(w + p.total);
+  cudaError_t e = cudaMemsetAsync(err, 0, 2 * sizeof(int), st);
   if (e != cudaSuccess) return e;
-
-  CUtensorMap mq, mx;
-  if (!make_map(&mq, qb, nq, pitch, kTcM) || !make_map(&mx, xb, n, pitch, kTcN)) return cudaErrorNotSupported;
-  TcArgs ta;
-  ta.xnorm = xnorm;
-  ta.n = n;
-  ta.nq = nq;
-  ta.kchunks = pitch / kTcK;
-  ta.cand = cand;
-  ta.slice = ((n + ns - 1) / ns + kTcN - 1) / kTcN * kTcN;
-  ta.nslice = ns;
-  ta.out = cand_buf;
-  ta.err = err_flag;
-  // as many ring stages as fit beside the candidate lists (at least 2, at most kMaxStages);
-  // one CTA per SM either way (the two accumulators take all 512 tensor-memory columns)
-  int maxsm = 0;
-  cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, knn_tc_kernel);
+  e = run_tc<true>(p, X, n, d, Q, nq, k, ids_out, dists_out, w, err, left_count, left, sms, st);
   if (e != cudaSuccess) return e;
-  maxsm -= (int)fa.sharedSizeBytes;  // the kernel's static shared memory comes off the top
-  const size_t fixed = 1024 + (size_t)cand * kEpiThreads * 8 + (2 * kMaxStages + 4) * 8 + 16;
-  int stages = kMaxStages;
-  while (stages > 2 && fixed + (size_t)stages * (kABytes + kBBytes) > (size_t)maxsm) --stages;
-  size_t smem = fixed + (size_t)stages * (kABytes + kBBytes);
-  if (smem > (size_t)maxsm) return cudaErrorInvalidConfiguration;
-  const size_t one_per_sm = ((size_t)maxsm + fa.sharedSizeBytes) / 2 + 1024;  // never two CTAs on one SM
-  if (smem < one_per_sm) smem = one_per_sm;
-  ta.stages = stages;
-  e = cudaFuncSetAttribute(knn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)((nq + kTcM - 1) / kTcM), (unsigned)ns);
-  knn_tc_kernel<<<grid, kTcThreads, smem, st>>>(mq, mx, ta);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-
-  const int ncand = ns * cand;
-  int P = 1;
-  while (P < ncand) P <<= 1;
-  const size_t fsm = (size_t)P * 8 * kFinWarps;
-  e = cudaFuncSetAttribute(knn_tc_finalize, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
-  if (e != cudaSuccess) return e;
-  long long fg = (nq + kFinWarps - 1) / kFinWarps;
-  if (fg > (long long)sms * 8) fg = (long long)sms * 8;
-  knn_tc_finalize<<<(unsigned)fg, kFinWarps * 32, fsm, st>>>(X, Q, nq, d, cand_buf, ncand, P, k, ids_out,
-                                                             dists_out);
-  return cudaGetLastError();
+  return launch_knn(X, n, d, Q, nq, k, ids_out, dists_out, ffma_scratch, st, left, left_count);
 }
 
 cudaError_t launch_bounded_wait_probe(long long limit_ns, int* gave_up, cudaStream_t st) {
