@@ -279,6 +279,31 @@ __device__ __forceinline__ void gather_batch(const float4* __restrict__ q4, cons
   }
 }
 
+// Insertion position of (dist, id) in the sorted list R for every lane at once, fixed steps on
+// the distances alone; equal distances (any lane's) are settled by id.  `keep` (in: this
+// lane has a candidate) is cleared when R already holds it.  Warp-wide.
+__device__ __forceinline__ int list_position(const float* s_rd, const int32_t* s_ri, int len, float dist, int32_t id,
+                                             bool& keep) {
+  int pos = 0;
+  for (int step = 1 << (31 - __clz(len)); step > 0; step >>= 1) {
+    const int t = pos + step;
+    if (t <= len && s_rd[t - 1] < dist) pos = t;
+  }
+  const bool tie = keep && pos < len && s_rd[pos] == dist;
+  if (__any_sync(kFull, tie) && tie) {
+    int lo = pos, hi = len;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      const bool less = s_rd[mid] == dist && (s_ri[mid] & ~kExpanded) < id;
+      if (less) lo = mid + 1; else hi = mid;
+    }
+    pos = lo;
+    keep = !(lo < len && s_rd[lo] == dist && (s_ri[lo] & ~kExpanded) == id);
+  }
+  __syncwarp();
+  return pos;
+}
+
 #ifdef PEOS_CHECKED
 // The list invariant after a merge: strictly ascending (dist, id), no id twice.
 static __device__ __noinline__ void check_list(const float* s_rd, const int32_t* s_ri, int len, int lane,
@@ -311,6 +336,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32, Shape<G>::kMinCtas) search_ker
   // lane (measured faster for them)
   constexpr bool kGroups = (NR == 2 && W == 1 && ROUTING != 0);
   constexpr int NL = kGroups ? 1 : NR;  // edges held per lane
+  // lists of up to 64 entries: the candidates' positions by a search of fixed steps (PEOs,
+  // where few lanes hold a candidate: sift-shaped 440 -> 432 us, GIST-shaped 2.85 -> 2.65 ms;
+  // plain routing 404 -> 444 us, and lists of 512 7.41 -> 7.82 ms, keep the divergent search)
+  constexpr bool kFixedSearch = W == 1 && NL == 1 && ROUTING != 0;
   constexpr int NRC = W * NL;     // candidate registers per lane: candidate g = r * 32 + lane
   [[maybe_unused]] constexpr int kCand = NRC * 32;  // candidates one iteration can hold (checked builds)
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -724,36 +753,46 @@ __global__ void __launch_bounds__(kMaxWarps * 32, Shape<G>::kMinCtas) search_ker
         gather_batch<kGather, NRC, DT>(q4, a.X, a.scales, d4, s_cid, b, min(kGather, npass - b), lane, mydist);
       c_ndist += npass;
 
-      // ---- candidates that can enter R: below the list bound (or the list is not full)
-      //      and not already in R (a node forgotten by the visited table); for each,
-      //      its insertion position in R by binary search on (dist, id)
+      // ---- candidates that can enter R: below the list bound (+inf while the list is not
+      //      full) and not already in R (a node forgotten by the visited table); for each,
+      //      its insertion position in R by (dist, id)
       uint64_t key[NRC];
       int pos[NRC];
       unsigned km[NRC];  // kept candidates of each register: bit `lane` = this lane's
       int nkeep = 0;
+      if (kFixedSearch && ef <= 64) {
+        const bool below = lane < npass && mydist[0] < delta2;
+        bool keep = below;
+        key[0] = below ? pack_key(mydist[0], s_cid[lane]) : kNoKey;
+        if (!__any_sync(kFull, below)) continue;
+        pos[0] = list_position(s_rd, s_ri, len, mydist[0], key_id(key[0]), keep);
+        km[0] = __ballot_sync(kFull, keep);
+        nkeep = __popc(km[0]);
+      } else {
 #pragma unroll
-      for (int r = 0; r < NRC; ++r) {
-        const int g = r * 32 + lane;
-        key[r] = kNoKey;
-        pos[r] = 0;
-        bool keep = false;
-        if (g < npass && (!full || mydist[r] < delta2)) {
-          const float kd = mydist[r];
-          const int32_t kid = s_cid[g];
-          key[r] = pack_key(kd, kid);
-          int lo = 0, hi = len;
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            const float md = s_rd[mid];
-            const int32_t mi = s_ri[mid] & ~kExpanded;
-            const bool less = (md < kd) || (md == kd && mi < kid);
-            if (less) lo = mid + 1; else hi = mid;
+        for (int r = 0; r < NRC; ++r) {
+          const int g = r * 32 + lane;
+          key[r] = kNoKey;
+          pos[r] = 0;
+          bool keep = false;
+          if (g < npass && mydist[r] < delta2) {
+            const float kd = mydist[r];
+            const int32_t kid = s_cid[g];
+            key[r] = pack_key(kd, kid);
+            int lo = 0, hi = len;
+            while (lo < hi) {
+              const int mid = (lo + hi) >> 1;
+              const float md = s_rd[mid];
+              const int32_t mi = s_ri[mid] & ~kExpanded;
+              const bool less = (md < kd) || (md == kd && mi < kid);
+              if (less) lo = mid + 1; else hi = mid;
+            }
+            pos[r] = lo;
+            keep = !(lo < len && s_rd[lo] == kd && (s_ri[lo] & ~kExpanded) == kid);
           }
-          pos[r] = lo;
-          keep = !(lo < len && s_rd[lo] == kd && (s_ri[lo] & ~kExpanded) == kid);
+          km[r] = __ballot_sync(kFull, keep);
+          nkeep += __popc(km[r]);
         }
-        km[r] = __ballot_sync(kFull, keep);
-        nkeep += __popc(km[r]);
       }
       if (nkeep == 0) continue;
 
@@ -774,15 +813,103 @@ __global__ void __launch_bounds__(kMaxWarps * 32, Shape<G>::kMinCtas) search_ker
         //      candidate before it did and dist < the (ef-1-g)-th entry of R (entries past
         //      len count as +inf); J = number entering
         const bool keep0 = (km[0] >> lane) & 1u;
-        int fail_rank = 0x7fffffff;
+        bool enters = false;
         if (keep0) {
           const int idx = ef - 1 - rank;
           const float bound = idx < 0 ? -INFINITY : (idx < len ? s_rd[idx] : INFINITY);
-          if (!(key_dist(key[0]) < bound)) fail_rank = rank;
+          enters = key_dist(key[0]) < bound;
         }
-        J = min(nkeep, __reduce_min_sync(kFull, fail_rank));
+        J = __popc(__ballot_sync(kFull, enters));  // the first J by rank: the bound falls as the rank grows
         if (J == 0) continue;
-        if (keep0 && rank < J) {
+        if (ef <= 64) {
+          // ---- merge of a short list: F = the slots the candidates take (position + rank); a
+          //      slot o before the list's new end that is not among them takes the entry
+          //      o - (slots of F below o).  One round trip to shared memory; staging the
+          //      candidates there and searching them for every entry took 457 us against 440
+          //      (sift-shaped PEOs, 10,000 queries; plain routing 420 against 404)
+          const int f = pos[0] + rank;
+          const unsigned flo = __reduce_or_sync(kFull, enters && f < 32 ? 1u << f : 0u);
+          const unsigned fhi = ef > 32 ? __reduce_or_sync(kFull, enters && f >= 32 ? 1u << (f - 32) : 0u) : 0u;
+          const unsigned under = (1u << lane) - 1u;
+          const int p0 = flo ? __ffs(flo) - 1 : __ffs(fhi) + 31;
+          len = min(ef, len + J);
+          const bool t0 = lane > p0 && lane < len && !((flo >> lane) & 1u);
+          const bool t1 = lane + 32 > p0 && lane + 32 < len && !((fhi >> lane) & 1u);
+          const int j0 = lane - __popc(flo & under), j1 = lane + 32 - __popc(flo) - __popc(fhi & under);
+          float d0 = 0.0f, d1 = 0.0f;
+          int32_t x0 = 0, x1 = 0;
+          if (t0) {
+            d0 = s_rd[j0];
+            x0 = s_ri[j0];
+          }
+          if (t1) {
+            d1 = s_rd[j1];
+            x1 = s_ri[j1];
+          }
+          __syncwarp();
+          if (t0) {
+            s_rd[lane] = d0;
+            s_ri[lane] = x0;
+          }
+          if (t1) {
+            s_rd[lane + 32] = d1;
+            s_ri[lane + 32] = x1;
+          }
+          if (enters && PEOS_EXPECT(f >= 0 && f < ef, kChkListWrite)) {
+            s_rd[f] = key_dist(key[0]);
+            s_ri[f] = key_id(key[0]);
+          }
+          hint = min(hint, p0);
+          c_ins += J;
+          __syncwarp();
+#ifdef PEOS_CHECKED
+          check_list(s_rd, s_ri, len, lane, a.check);
+#endif
+          continue;
+        }
+        if constexpr (kFixedSearch) {
+          // ---- merge of a longer list: the same, 32 slots at a time from the list's new end
+          //      down to the first slot taken (a slot's source lies at or below it, so the
+          //      slots written so far are not read again).  PEOs, uneven lists of up to 512:
+          //      7.46 -> 7.16 ms; plain routing keeps the staged form below (with this code
+          //      beside it its short lists ran 404 -> 451 us)
+          const int f = pos[0] + rank;
+          const int p0 = __reduce_min_sync(kFull, enters ? f : 0x7fffffff);
+          const int end = min(ef, len + J);
+          int under_end = J;  // slots taken below the current 32
+          for (int c = (end - 1) >> 5; c >= p0 >> 5; --c) {
+            const unsigned F = __reduce_or_sync(kFull, enters && (f >> 5) == c ? 1u << (f & 31) : 0u);
+            under_end -= __popc(F);
+            const int o = 32 * c + lane;
+            const int j = o - under_end - __popc(F & ((1u << lane) - 1u));
+            const bool takes = o > p0 && o < end && !((F >> lane) & 1u);
+            float dd = 0.0f;
+            int32_t ii = 0;
+            if (takes) {
+              dd = s_rd[j];
+              ii = s_ri[j];
+            }
+            __syncwarp();
+            if (takes && PEOS_EXPECT(j >= 0 && j < o, kChkListWrite)) {
+              s_rd[o] = dd;
+              s_ri[o] = ii;
+            }
+            __syncwarp();
+          }
+          if (enters && PEOS_EXPECT(f >= 0 && f < ef, kChkListWrite)) {
+            s_rd[f] = key_dist(key[0]);
+            s_ri[f] = key_id(key[0]);
+          }
+          len = end;
+          hint = min(hint, p0);
+          c_ins += J;
+          __syncwarp();
+#ifdef PEOS_CHECKED
+          check_list(s_rd, s_ri, len, lane, a.check);
+#endif
+          continue;
+        }
+        if (enters) {
           s_ckey[rank] = key[0];
           s_cpos[rank] = pos[0];
         }
