@@ -477,7 +477,7 @@ peos_status peos_build_codes_permuted(const peos_graph* graph, const peos_matrix
       for (int j = 0; j < m; ++j) hW16[(size_t)t * pv + j] = hW[(size_t)t * m + j];
   }
   const size_t w16 = hW16.size() * sizeof(float);
-  const size_t sb = build_codes_scratch_bytes(n, L, m);
+  const size_t sb = build_codes_scratch_bytes(n, d, L, m);
   StreamScratch scratch(s);
   if (e == cudaSuccess && sb + w16 > 0) e = scratch.alloc(((sb + 255) & ~(size_t)255) + w16);
   const float* W16 = c->Wt;
@@ -491,8 +491,9 @@ peos_status peos_build_codes_permuted(const peos_graph* graph, const peos_matrix
     e = launch_node_proj(static_cast<const float*>(base->data), n, d, L, m, c->A, c->B, W16, c->perm, c->node_proj,
                          table_stride(L, m), c->norms, s);
   if (e == cudaSuccess)
-    e = launch_build_codes(static_cast<const float*>(base->data), n, d, graph->nbrs, R, L, m, c->A, c->B, W16, c->perm,
-                           c->node_proj, table_stride(L, m), c->records, c->rec_stride, scratch.p, s);
+    e = launch_build_codes(static_cast<const float*>(base->data), n, d, graph->nbrs, R, L, m, c->A, c->B, W16,
+                           m < pv ? hW16.data() : hW.data(), c->perm, c->node_proj, table_stride(L, m), c->records,
+                           c->rec_stride, scratch.p, s);
   // the host vectors hA/hB go out of scope: wait for their copies
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {

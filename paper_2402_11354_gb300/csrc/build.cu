@@ -10,10 +10,15 @@
 // kernels: a thread takes whole edges (or rows) and all 16 sums of each, so that a vector
 // element read from shared memory serves several edges.  For larger m one CTA per node
 // with a thread per sum (node_proj_kernel, build_codes_kernel).
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <math.h>
+
+#include <string.h>
 
 #include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "device.cuh"
 #include "internal.h"
@@ -308,6 +313,10 @@ struct TileArgs {
   uint8_t* rec;
   size_t rec_stride;
   int bits, cpw, nwords;
+  // edges, screened form
+  const uint4* frag;    // the vectors as MMA fragments: [L][ksteps][4][32] {hi, hi, lo, lo}
+  const float* amax;    // [L + 1] largest ||a^i_j|| of block i over j; last: largest ||b_j||_i over j, i
+  int ksteps;           // steps of 16 coordinates per block
   float2* blocks;       // per warp: {squared block norm, code} of the tile's edges, [L][kEdgeTile]
   int* work;
 };
@@ -475,36 +484,26 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) node_rows_kernel(TileArgs 
   }
 }
 
-// Edge records.  Per tile of 128 edges two passes over the coordinates: the a^i sums and
-// the block norms (their codes and squared norms go to `blocks`), then, the block norms'
-// mean being known, the b_j sums of e_res.
-template <int KU, bool PERM, bool WSMEM>
-__global__ void __launch_bounds__(kTileWarps * 32, 1) build_edges_kernel(TileArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4* s_w = reinterpret_cast<float4*>(smem_raw);
-  const float4* w = tile_vectors<WSMEM>(a, s_w);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kQueue = kEdgeTile + 32;
-  constexpr size_t kWarpBytes = (size_t)kEdgeTile * kTilePitch * 16 + (size_t)kQueue * 12;
-  unsigned char* base =
-      reinterpret_cast<unsigned char*>(s_w + (WSMEM ? 2 * a.d * (kVecs / 4) : 0)) + (size_t)warp * kWarpBytes;
-  float4* s_e = reinterpret_cast<float4*>(base);
-  int32_t* q_u = reinterpret_cast<int32_t*>(base + (size_t)kEdgeTile * kTilePitch * 16);
-  int32_t* q_v = q_u + kQueue;
-  int32_t* q_s = q_v + kQueue;
-  const int d = a.d, L = a.L, m = a.m, dp = d / L, R = a.R;
-  float2* blk = a.blocks + ((size_t)blockIdx.x * kTileWarps + warp) * L * kEdgeTile;
-  const size_t ids_end = rec_ids_offset(R) + 4 * (size_t)R, codes_at = rec_codes_offset(R);
-  const size_t used = codes_at + 8 * (size_t)a.nwords * R;
-  const int gap4 = (int)(codes_at - ids_end) / 4, pad4 = (int)(a.rec_stride - used) / 4;
-
+// A warp's queue of valid edges, filled in slot order from the nodes it takes: the slots'
+// ids go to the records and empty slots are zeroed on the way.
+template <int TILE>
+struct EdgeQueue {
+  static constexpr int kSlots = TILE + 32;
+  int32_t *u, *v, *s;     // [kSlots] in shared memory: neighbour, node, slot
   long long v0 = 0;       // the chunk's first node
   int slots = 0, at = 0;  // its slots, and how many are queued or written
-  bool more = true;
   int queued = 0;
-  for (;;) {
-    // ---- fill the queue: the slots' ids go to the records, empty slots are zeroed
-    while (queued < kEdgeTile && more) {
+  bool more = true;
+
+  __device__ __forceinline__ explicit EdgeQueue(int32_t* mem) : u(mem), v(mem + kSlots), s(mem + 2 * kSlots) {}
+
+  // at least TILE edges, or all that are left; the tile's edges (warp-wide)
+  __device__ __forceinline__ int fill(const TileArgs& a, int lane) {
+    const int R = a.R;
+    const size_t ids_end = rec_ids_offset(R) + 4 * (size_t)R, codes_at = rec_codes_offset(R);
+    const size_t used = codes_at + 8 * (size_t)a.nwords * R;
+    const int gap4 = (int)(codes_at - ids_end) / 4, pad4 = (int)(a.rec_stride - used) / 4;
+    while (queued < TILE && more) {
       if (at >= slots) {
         int c = 0;
         if (lane == 0) c = atomicAdd(a.work, 1);
@@ -517,38 +516,83 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) build_edges_kernel(TileArg
         slots = nn * R;
         at = 0;
         for (int t = lane; t < nn * (gap4 + pad4); t += 32) {
-          const int v = t / (gap4 + pad4), b = t - v * (gap4 + pad4);
-          uint8_t* r = a.rec + (size_t)(v0 + v) * a.rec_stride;
+          const int w = t / (gap4 + pad4), b = t - w * (gap4 + pad4);
+          uint8_t* r = a.rec + (size_t)(v0 + w) * a.rec_stride;
           *reinterpret_cast<uint32_t*>(b < gap4 ? r + ids_end + 4 * b : r + used + 4 * (b - gap4)) = 0u;
         }
       }
       const int t = at + lane;
-      int32_t u = -1, s = 0;
-      long long v = v0;
+      int32_t id = -1;
+      int slot = 0;
+      long long node = v0;
       if (t < slots) {
-        u = __ldg(a.nbrs + (size_t)v0 * R + t);
+        id = __ldg(a.nbrs + (size_t)v0 * R + t);
         const int lv = t / R;
-        v = v0 + lv;
-        s = t - lv * R;
-        uint8_t* r = a.rec + (size_t)v * a.rec_stride;
-        reinterpret_cast<int32_t*>(r + rec_ids_offset(R))[s] = u;
-        if (u < 0) {
-          reinterpret_cast<float4*>(r)[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int k = 0; k < a.nwords; ++k) reinterpret_cast<uint64_t*>(r + codes_at)[(size_t)k * R + s] = 0;
+        node = v0 + lv;
+        slot = t - lv * R;
+        uint8_t* r = a.rec + (size_t)node * a.rec_stride;
+        reinterpret_cast<int32_t*>(r + rec_ids_offset(R))[slot] = id;
+        if (id < 0) {
+          reinterpret_cast<float4*>(r)[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int k = 0; k < a.nwords; ++k) reinterpret_cast<uint64_t*>(r + codes_at)[(size_t)k * R + slot] = 0;
         }
       }
-      const unsigned have = __ballot_sync(kFull, u >= 0);
-      if (u >= 0) {
+      const unsigned have = __ballot_sync(kFull, id >= 0);
+      if (id >= 0) {
         const int p = queued + __popc(have & ((1u << lane) - 1u));
-        q_u[p] = u;
-        q_v[p] = (int32_t)v;
-        q_s[p] = s;
+        u[p] = id;
+        v[p] = (int32_t)node;
+        s[p] = slot;
       }
       queued += __popc(have);
       at += 32;
     }
     __syncwarp();
-    const int cnt = min(queued, kEdgeTile);
+    return min(queued, TILE);
+  }
+
+  // the tile is done: the rest moves to the front
+  __device__ __forceinline__ void drop(int cnt, int lane) {
+    const int rest = queued - cnt;
+    int32_t ru = 0, rv = 0, rs = 0;
+    __syncwarp();
+    if (lane < rest) {
+      ru = u[cnt + lane];
+      rv = v[cnt + lane];
+      rs = s[cnt + lane];
+    }
+    __syncwarp();
+    if (lane < rest) {
+      u[lane] = ru;
+      v[lane] = rv;
+      s[lane] = rs;
+    }
+    queued = rest;
+  }
+};
+
+// Edge records.  Per tile of 64 edges two passes over the coordinates: the a^i sums and
+// the block norms (their codes and squared norms go to `blocks`), then, the block norms'
+// mean being known, the b_j sums of e_res.
+template <int KU, bool PERM, bool WSMEM>
+__global__ void __launch_bounds__(kTileWarps * 32, 1) build_edges_kernel(TileArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float4* s_w = reinterpret_cast<float4*>(smem_raw);
+  const float4* w = tile_vectors<WSMEM>(a, s_w);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  using Queue = EdgeQueue<kEdgeTile>;
+  constexpr size_t kWarpBytes = (size_t)kEdgeTile * kTilePitch * 16 + (size_t)Queue::kSlots * 12;
+  unsigned char* base =
+      reinterpret_cast<unsigned char*>(s_w + (WSMEM ? 2 * a.d * (kVecs / 4) : 0)) + (size_t)warp * kWarpBytes;
+  float4* s_e = reinterpret_cast<float4*>(base);
+  Queue queue(reinterpret_cast<int32_t*>(base + (size_t)kEdgeTile * kTilePitch * 16));
+  const int32_t *q_u = queue.u, *q_v = queue.v, *q_s = queue.s;
+  const int d = a.d, L = a.L, m = a.m, dp = d / L, R = a.R;
+  float2* blk = a.blocks + ((size_t)blockIdx.x * kTileWarps + warp) * L * kEdgeTile;
+  const size_t codes_at = rec_codes_offset(R);
+
+  for (;;) {
+    const int cnt = queue.fill(a, lane);
     if (cnt == 0) break;
 
     auto stage = [&](int c0) {
@@ -685,22 +729,353 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) build_edges_kernel(TileArg
         *cwords = *cwords | (uint64_t)(sel & 0xffff) | ((uint64_t)(sel >> 16) << (a.bits - 1));
       }
     }
-    // ---- the queue's rest moves to the front
-    const int rest = queued - cnt;
-    int32_t ru = 0, rv = 0, rs = 0;
-    __syncwarp();
-    if (lane < rest) {
-      ru = q_u[cnt + lane];
-      rv = q_v[cnt + lane];
-      rs = q_s[cnt + lane];
+    queue.drop(cnt, lane);
+  }
+}
+
+// ---- the screened form: blocks of 8..64 coordinates, a multiple of 4 -----------------
+//
+// A code is an argmax over 16 sums, and only that: sums good to five digits settle all but a
+// few in a thousand.  A warp takes 32 edges and forms, on the tensor cores, every e_i . a^i_j
+// and e_i . b_j (two BF16 terms of each factor, three products, mma.sync on fragments built
+// straight from the staged rows); per block it keeps the two largest |e_i . a^i_j|, and the
+// b_j sums of e_res follow from two running sums, sum_i P_i and sum_i P_i / ||e_i||, since
+// block i of e_res is e_i (1 - mean / ||e_i||).  Where the two largest are closer than the
+// error bound of both the estimate and the sequential FP32 sum, the 16 sums are formed again
+// in that order and decide, so the codes are those of the tiled form bit for bit.  The block
+// norms are sequential FP32 sums as there (a lane per edge).
+constexpr int kScreenWarps = 16;  // one CTA per SM
+constexpr int kScreenDims = 64;   // coordinates staged at a time: whole blocks, at most this many
+constexpr int kMaxCoef = 96;      // blocks per edge (L <= 95, see kMaxCodeWords)
+
+// coordinates staged at a time and the staged row's pitch in 16-byte units: odd, so that
+// neither a lane per row nor four lanes per row meet a bank conflict
+__host__ __device__ inline int screen_dims(int dp) { return dp * (kScreenDims / dp); }
+__host__ __device__ inline int screen_pitch(int dp) { return (screen_dims(dp) / 4) | 1; }
+size_t screen_warp_bytes(int dp) {
+  return (size_t)32 * screen_pitch(dp) * 16 + (size_t)EdgeQueue<32>::kSlots * 12 + (size_t)kMaxCoef * 4;
+}
+
+__device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+// hi and lo BF16 terms of four values, as two packed pairs each
+__device__ __forceinline__ void split4(const float4& x, uint32_t (&hi)[2], uint32_t (&lo)[2]) {
+  hi[0] = bf16x2(x.x, x.y);
+  hi[1] = bf16x2(x.z, x.w);
+  lo[0] = bf16x2(x.x - __uint_as_float(hi[0] << 16), x.y - __uint_as_float(hi[0] & 0xffff0000u));
+  lo[1] = bf16x2(x.z - __uint_as_float(hi[1] << 16), x.w - __uint_as_float(hi[1] & 0xffff0000u));
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// The two largest of a row's 16 values |p_j|, as keys: the value's bits with the low five
+// replaced by (j, sign).  A quad of lanes holds four rows, four values of each per lane;
+// lane c of the quad gets row c's result.
+struct Top2 {
+  uint32_t first, second;
+};
+__device__ __forceinline__ uint32_t top_key(float p, int j) {
+  const uint32_t b = __float_as_uint(p);
+  return (b & 0x7fffffe0u) | (uint32_t)(2 * j) | (b >> 31);
+}
+__device__ __forceinline__ Top2 top_merge(const Top2& x, const Top2& y) {
+  return Top2{max(x.first, y.first), max(min(x.first, y.first), max(x.second, y.second))};
+}
+__device__ __forceinline__ Top2 quad_top2(const float (&row)[4][4], int t) {
+  // row[q][i]: value i of row q on this lane; columns 2t, 2t + 1, 8 + 2t, 9 + 2t
+  Top2 m[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint32_t a = top_key(row[q][0], 2 * t), b = top_key(row[q][1], 2 * t + 1), c = top_key(row[q][2], 2 * t + 8),
+                   d = top_key(row[q][3], 2 * t + 9);
+    m[q] = top_merge(Top2{max(a, b), min(a, b)}, Top2{max(c, d), min(c, d)});
+  }
+  // lanes t and t ^ 2 share rows {0, 1} / {2, 3}, then t and t ^ 1 one row each
+  const bool up2 = t & 2, up1 = t & 1;
+  Top2 k[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const Top2 keep = up2 ? m[q + 2] : m[q], give = up2 ? m[q] : m[q + 2];
+    const Top2 got{__shfl_xor_sync(kFull, give.first, 2), __shfl_xor_sync(kFull, give.second, 2)};
+    k[q] = top_merge(keep, got);
+  }
+  const Top2 keep = up1 ? k[1] : k[0], give = up1 ? k[0] : k[1];
+  const Top2 got{__shfl_xor_sync(kFull, give.first, 1), __shfl_xor_sync(kFull, give.second, 1)};
+  return top_merge(keep, got);
+}
+// settled: the largest is ahead of the second by more than twice the bound on a value's error
+// (and the keys' own truncation), so it is the argmax and has the sign of its estimate
+__device__ __forceinline__ bool top_settled(const Top2& k, float err) {
+  const float v1 = __uint_as_float(k.first & 0x7fffffe0u), v2 = __uint_as_float(k.second & 0x7fffffe0u);
+  return v1 - v2 > 2.0f * err + v1 * 0x1p-17f;
+}
+__device__ __forceinline__ int top_code(const Top2& k) { return (int)((k.first >> 1) & 15u) | (int)((k.first & 1u) << 16); }
+
+// argmax over the sums p_j of lanes j = 0..15, as argmax16 (warp-wide; the result on every lane)
+__device__ __forceinline__ int lanes_argmax(float p) {
+  float pv = __shfl_sync(kFull, p, 0), bv = fabsf(pv);
+  int best = 0;
+  for (int j = 1; j < kVecs; ++j) {
+    const float x = __shfl_sync(kFull, p, j), ax = fabsf(x);
+    if (ax > bv) {
+      bv = ax;
+      pv = x;
+      best = j;
     }
-    __syncwarp();
-    if (lane < rest) {
-      q_u[lane] = ru;
-      q_v[lane] = rv;
-      q_s[lane] = rs;
+  }
+  return best | ((pv >= 0.0f) ? 0 : 1 << 16);
+}
+
+template <bool PERM, bool FSMEM>
+__global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_kernel(TileArgs a, float c_a, float c_b,
+                                                                                   float c_fp) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 3;
+  const int d = a.d, L = a.L, m = a.m, dp = d / L, R = a.R, KS = a.ksteps;
+  const int pitch = screen_pitch(dp), cd = screen_dims(dp);
+  const uint4* frag = a.frag;
+  unsigned char* mem = smem_raw;
+  if (FSMEM) {
+    uint4* f = reinterpret_cast<uint4*>(smem_raw);
+    const int nf = L * KS * 4 * 32;
+    for (int i = threadIdx.x; i < nf; i += blockDim.x) f[i] = __ldg(a.frag + i);
+    __syncthreads();
+    frag = f;
+    mem += (size_t)nf * 16;
+  }
+  mem += (size_t)warp * ((size_t)32 * pitch * 16 + (size_t)EdgeQueue<32>::kSlots * 12 + (size_t)kMaxCoef * 4);
+  float4* s_e = reinterpret_cast<float4*>(mem);
+  EdgeQueue<32> queue(reinterpret_cast<int32_t*>(mem + (size_t)32 * pitch * 16));
+  float* s_coef = reinterpret_cast<float*>(mem + (size_t)32 * pitch * 16 + (size_t)EdgeQueue<32>::kSlots * 12);
+  const float* rows = reinterpret_cast<const float*>(s_e);
+  const size_t codes_at = rec_codes_offset(R);
+  const float bmax = __ldg(a.amax + L);
+
+  // lane l owns edge l of the tile; in the MMA fragments edge 4 r + 2 mt + h is row 8 h + r of
+  // the mt-th 16-row tile (r = 0..7), so a quad's four rows belong to its four lanes
+  for (;;) {
+    const int cnt = queue.fill(a, lane);
+    if (cnt == 0) break;
+    const bool have = lane < cnt;
+    const int32_t u = have ? queue.u[lane] : 0, v = have ? queue.v[lane] : 0;
+    const int slot = have ? queue.s[lane] : 0;
+    if (!PERM) {  // the rows' later lines come into L2 while the first coordinates are worked on
+      const int lines = (d * 4 + 127) >> 7;
+      if (have)
+        for (int l = 0; l < lines; ++l) {
+          const char* p = reinterpret_cast<const char*>(a.X + (size_t)u * d) + ((size_t)l << 7);
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+        }
     }
-    queued = rest;
+    uint8_t* rec = a.rec + (size_t)v * a.rec_stride;
+    uint64_t* cwords = reinterpret_cast<uint64_t*>(rec + codes_at) + slot;
+    const float* tv = a.node_proj + (size_t)v * a.proj_stride;
+
+    float tot2 = 0.0f, sum = 0.0f, h1 = 0.0f, pending = 0.0f;
+    uint64_t word = 0;
+    int wk = 1, wi = 0;
+    float S1[4][4], S2[4][4];  // [row of the quad][value]: sum_i P_i and sum_i P_i / ||e_i||
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int x = 0; x < 4; ++x) S1[q][x] = S2[q][x] = 0.0f;
+
+    bool tiny = false;  // a block whose squared norm loses its precision: e[0] is settled in order
+    int i = 0;          // the block
+    for (int c0 = 0; c0 < d; c0 += cd) {
+      const int cw4 = min(cd, d - c0) >> 2;
+      __syncwarp();
+      {
+        // 32 rows of cw4 pieces, a piece per lane and step
+        const int dr = 32 / cw4, dc = 32 - dr * cw4;
+        int e = lane / cw4, col = lane - e * cw4;
+#pragma unroll 4
+        for (int j = 0; j < cw4; ++j) {
+          if (e < cnt) {
+            const float4 x = row4<PERM>(a.X, queue.u[e], d, c0 + 4 * col, a.perm);
+            const float4 y = row4<PERM>(a.X, queue.v[e], d, c0 + 4 * col, a.perm);
+            s_e[e * pitch + col] = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
+          }
+          e += dr;
+          col += dc;
+          if (col >= cw4) {
+            col -= cw4;
+            ++e;
+          }
+        }
+      }
+      __syncwarp();
+#pragma unroll 1
+      for (int b0 = 0; b0 < cw4 * 4; b0 += dp, ++i) {
+        // block norm of the lane's own edge, in order
+        float n2 = 0.0f;
+        uint32_t any = 0;
+        for (int k = 0; k < dp; k += 4) {
+          const float4 x = s_e[lane * pitch + ((b0 + k) >> 2)];
+          n2 = n2 + x.x * x.x;
+          n2 = n2 + x.y * x.y;
+          n2 = n2 + x.z * x.z;
+          n2 = n2 + x.w * x.w;
+          any |= __float_as_uint(x.x) | __float_as_uint(x.y) | __float_as_uint(x.z) | __float_as_uint(x.w);
+        }
+        const bool zero = (any & 0x7fffffffu) == 0u;  // every sum is 0: code +1
+        const bool small = !zero && !(n2 >= 1e-30f);
+        tiny = tiny || small;
+        const float bn = sqrtf(n2);
+        tot2 = tot2 + n2;
+        sum = sum + bn;
+        const float inv = bn > 0.0f ? __frcp_rn(bn) : 0.0f;
+        // P = e_i . (a^i_0..15, b_0..15)
+        float c[2][4][4];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) c[mt][nt][x] = 0.0f;
+        for (int ks = 0; ks < KS; ++ks) {
+          uint32_t hi[2][4], lo[2][4];
+          const bool in = 16 * ks + 4 * t < dp;
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int e = (lane & ~3) + 2 * mt + h;
+              const float4 x = in ? s_e[e * pitch + ((b0 + 16 * ks) >> 2) + t] : make_float4(0.f, 0.f, 0.f, 0.f);
+              uint32_t xh[2], xl[2];
+              split4(x, xh, xl);
+              hi[mt][h] = xh[0];
+              hi[mt][2 + h] = xh[1];
+              lo[mt][h] = xl[0];
+              lo[mt][2 + h] = xl[1];
+            }
+          const uint4* f = frag + ((size_t)(i * KS + ks) * 4) * 32 + lane;
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt) {
+            const uint4 w = FSMEM ? f[nt * 32] : __ldg(f + nt * 32);
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+              mma_bf16(c[mt][nt], hi[mt], w.x, w.y);
+              mma_bf16(c[mt][nt], lo[mt], w.x, w.y);
+              mma_bf16(c[mt][nt], hi[mt], w.z, w.w);
+            }
+          }
+        }
+        // row q = 2 mt + h of the quad: columns 2t, 2t + 1 of n-tiles 0, 1 (a) and 2, 3 (b)
+        float pa[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int mt = q >> 1, h = q & 1;
+          const float iq = __shfl_sync(kFull, inv, (lane & ~3) + q);
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            pa[q][x] = c[mt][x >> 1][2 * h + (x & 1)];
+            const float pb = c[mt][2 + (x >> 1)][2 * h + (x & 1)];
+            S1[q][x] = S1[q][x] + (iq != 0.0f ? pb : 0.0f);
+            S2[q][x] = fmaf(pb, iq, S2[q][x]);
+          }
+        }
+        const Top2 top = quad_top2(pa, t);
+        int sel = zero ? 0 : top_code(top);
+        const bool open = have && !zero && (small || !top_settled(top, c_a * __ldg(a.amax + i) * bn));
+        for (unsigned todo = __ballot_sync(kFull, open); todo; todo &= todo - 1) {
+          const int e = __ffs(todo) - 1;
+          float p = 0.0f;
+          if (lane < kVecs) {
+            const float* w = a.W + (size_t)(d + i * dp) * kVecs + lane;
+            for (int k = 0; k < dp; ++k) p = p + __ldg(w + (size_t)k * kVecs) * rows[(size_t)e * pitch * 4 + b0 + k];
+          }
+          const int got = lanes_argmax(p);
+          if (lane == e) sel = got;
+        }
+        // the code; its table entry is added a block later, when it has arrived
+        h1 = h1 + pending;
+        if (have) {
+          const float val = __ldg(tv + (i + 1) * m + (sel & 0xffff));
+          pending = (sel >> 16) ? -val : val;
+          word |= ((uint64_t)(sel & 0xffff) | ((uint64_t)(sel >> 16) << (a.bits - 1))) << (wk * a.bits);
+          if (++wk == a.cpw) {
+            cwords[(size_t)wi * R] = word;
+            word = 0;
+            wk = 0;
+            ++wi;
+          }
+        }
+      }
+    }
+    h1 = h1 + pending;
+    if (have && wk > 0) cwords[(size_t)wi * R] = word;
+    const float norm = sqrtf(tot2);
+    float wr = 1.0f, cr = 0.0f, mean = 0.0f;
+    if (norm != 0.0f) {
+      wr = sum / (sqrtf((float)L) * norm);
+      if (wr > 1.0f) wr = 1.0f;
+      cr = sqrtf((float)L) * sqrtf(fmaxf(0.0f, 1.0f - wr * wr));
+      mean = sum / (float)L;
+    }
+    // ---- e[0]: the sums of e_res with the b_j
+    float pb[4][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float mq = __shfl_sync(kFull, mean, (lane & ~3) + q);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) pb[q][x] = S1[q][x] - mq * S2[q][x];
+    }
+    const Top2 top = quad_top2(pb, t);
+    int sel0 = top_code(top);
+    // sum_i | ||e_i|| - mean | <= sqrt(L (sum ||e_i||^2 - L mean^2)), the weight of the estimates'
+    // errors; the two running sums and the sequential sum round relative to sum ||e_i||
+    const float spread = sqrtf((float)L * fmaxf(tot2 - sum * mean, 0.0f) + 1e-6f * (float)L * tot2);
+    const bool open = have && norm != 0.0f && (tiny || !top_settled(top, bmax * (c_b * spread + c_fp * sum)));
+    for (unsigned todo = __ballot_sync(kFull, open); todo; todo &= todo - 1) {
+      const int e = __ffs(todo) - 1;
+      const int32_t eu = queue.u[e], ev = queue.v[e];
+      const float em = __shfl_sync(kFull, mean, e);
+      float* lin = reinterpret_cast<float*>(s_e);  // the edge's d coordinates, in order
+      __syncwarp();
+      for (int k = 4 * lane; k < d; k += 128) {
+        const float4 x = row4<PERM>(a.X, eu, d, k, a.perm), y = row4<PERM>(a.X, ev, d, k, a.perm);
+        *reinterpret_cast<float4*>(lin + k) = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
+      }
+      __syncwarp();
+      for (int i = lane; i < L; i += 32) {
+        float n2 = 0.0f;
+        for (int k = 0; k < dp; ++k) n2 = n2 + lin[i * dp + k] * lin[i * dp + k];
+        const float b = sqrtf(n2);
+        s_coef[i] = (b > 0.0f) ? (1.0f - em / b) : 0.0f;
+      }
+      __syncwarp();
+      float p = 0.0f;
+      if (lane < kVecs) {
+        const float* w = a.W + lane;
+        for (int i = 0; i < L; ++i) {
+          const float cf = s_coef[i];
+#pragma unroll 4
+          for (int k = i * dp; k < (i + 1) * dp; ++k) p = p + __ldg(w + (size_t)k * kVecs) * (lin[k] * cf);
+        }
+      }
+      const int got = lanes_argmax(p);
+      if (lane == e) sel0 = got;
+    }
+    if (have) {
+      if (norm == 0.0f) {  // a degenerate edge gets code +1 everywhere
+        sel0 = 0;
+        h1 = 0.0f;
+        for (int i = 0; i < L; ++i) h1 = h1 + __ldg(tv + (i + 1) * m);
+        for (int k = 0; k < a.nwords; ++k) cwords[(size_t)k * R] = 0;
+      }
+      const float v0f = __ldg(tv + (sel0 & 0xffff));
+      const float h2 = (sel0 >> 16) ? -v0f : v0f;
+      reinterpret_cast<float4*>(rec)[slot] = make_float4(norm, wr, cr, wr * h1 + cr * h2);
+      cwords[0] = cwords[0] | (uint64_t)(sel0 & 0xffff) | ((uint64_t)(sel0 >> 16) << (a.bits - 1));
+    }
+    queue.drop(cnt, lane);
   }
 }
 
@@ -863,19 +1238,95 @@ cudaError_t launch_tile_any(const TileArgs& a, int grid, cudaStream_t st) {
 
 int edges_grid(int64_t n) { return (int)std::min<int64_t>(num_sms(), (n + kNodeChunk - 1) / kNodeChunk); }
 
+bool screened(int d, int L, int m) {
+  const int dp = d / L;
+  return m <= kVecs && dp % 4 == 0 && dp >= 8 && dp <= kScreenDims && L < kMaxCoef && 32 * screen_pitch(dp) * 4 >= d;
+}
+
+// The fragment table and the norms of the screened form, from the k-major vectors W (2 d rows
+// of 16: the b_j, then the a^i_j).  Coordinate 4 t + x of a step of 16 sits where the MMA's
+// A fragment has lane t's x-th element.
+struct ScreenTables {
+  std::vector<uint32_t> frag;
+  std::vector<float> amax;
+};
+uint16_t host_bf16(float f) {  // round to nearest even (finite values)
+  uint32_t u;
+  memcpy(&u, &f, 4);
+  return (uint16_t)((u + 0x7fffu + ((u >> 16) & 1u)) >> 16);
+}
+float host_widen(uint16_t h) {
+  const uint32_t u = (uint32_t)h << 16;
+  float f;
+  memcpy(&f, &u, 4);
+  return f;
+}
+ScreenTables screen_tables(const float* W, int d, int L) {
+  const int dp = d / L, KS = (dp + 15) / 16;
+  ScreenTables T;
+  T.frag.assign((size_t)L * KS * 4 * 32 * 4, 0u);
+  T.amax.assign((size_t)L + 1, 0.0f);
+  auto at = [&](int i, int k, int col) -> float {  // column 0..15: a^i, 16..31: b
+    if (k >= dp) return 0.0f;
+    return col < 16 ? W[((size_t)d + (size_t)i * dp + k) * kVecs + col] : W[((size_t)i * dp + k) * kVecs + col - 16];
+  };
+  for (int i = 0; i < L; ++i) {
+    for (int col = 0; col < 32; ++col) {
+      double n2 = 0.0;
+      for (int k = 0; k < dp; ++k) n2 += (double)at(i, k, col) * at(i, k, col);
+      float& most = T.amax[col < 16 ? i : L];
+      most = std::max(most, (float)(sqrt(n2) * (1.0 + 1e-6)));
+    }
+    for (int ks = 0; ks < KS; ++ks)
+      for (int nt = 0; nt < 4; ++nt)
+        for (int lane = 0; lane < 32; ++lane) {
+          const int g = lane >> 2, t = lane & 3;
+          uint32_t* o = &T.frag[((((size_t)i * KS + ks) * 4 + nt) * 32 + lane) * 4];
+          for (int r = 0; r < 2; ++r) {
+            uint32_t hi = 0, lo = 0;
+            for (int x = 0; x < 2; ++x) {
+              const float v = at(i, 16 * ks + 4 * t + 2 * r + x, 8 * nt + g);
+              const uint16_t h = host_bf16(v), l = host_bf16(v - host_widen(h));
+              hi |= (uint32_t)h << (16 * x);
+              lo |= (uint32_t)l << (16 * x);
+            }
+            o[r] = hi;
+            o[2 + r] = lo;
+          }
+        }
+  }
+  return T;
+}
+
+template <bool PERM, bool FSMEM>
+cudaError_t launch_screened(const TileArgs& a, int grid, size_t smem, cudaStream_t st) {
+  auto fn = build_edges_screened_kernel<PERM, FSMEM>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // a value's error relative to ||a|| ||e_i||: three products of two-term BF16 factors (dropped
+  // and rounded terms 3.05 2^-16), their FP32 accumulation (2^-23 per product), and the
+  // sequential sum it stands for (2^-24 per coordinate, with the norms' own rounding)
+  const int dp = a.d / a.L;
+  const double c = 3.05 * 0x1p-16 + 48.0 * a.ksteps * 0x1p-23 + (2.0 * dp + 8.0) * 0x1p-24;
+  const double fp = (a.d + 2.0 * a.L + 16.0) * 0x1p-23;
+  fn<<<(unsigned)grid, kScreenWarps * 32, smem, st>>>(a, (float)(c * 1.01), (float)(c * 1.01), (float)fp);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 int codes_padded_vecs() { return kVecs; }
 
-size_t build_codes_scratch_bytes(int64_t n, int L, int m) {
+size_t build_codes_scratch_bytes(int64_t n, int d, int L, int m) {
   if (m > kVecs || n <= 0) return 0;
+  if (screened(d, L, m)) return 512 + (size_t)L * 4 + (size_t)L * ((d / L + 15) / 16) * 4 * 32 * 16;
   return 256 + (size_t)edges_grid(n) * kTileWarps * L * kEdgeTile * sizeof(float2);
 }
 
 cudaError_t launch_build_codes(const float* X, int64_t n, int d, const int32_t* nbrs, int R, int L, int m,
-                               const float* A, const float* B, const float* W16, const int32_t* perm,
-                               const float* node_proj, int proj_stride, uint8_t* rec, size_t rec_stride,
-                               void* scratch, cudaStream_t st) {
+                               const float* A, const float* B, const float* W16, const float* W16_host,
+                               const int32_t* perm, const float* node_proj, int proj_stride, uint8_t* rec,
+                               size_t rec_stride, void* scratch, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   if (m <= kVecs) {
     cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int), st);
@@ -898,6 +1349,26 @@ cudaError_t launch_build_codes(const float* X, int64_t n, int d, const int32_t* 
     a.cpw = codes_per_word(m);
     a.nwords = code_words(L, m);
     a.work = static_cast<int*>(scratch);
+    if (screened(d, L, m)) {
+      const ScreenTables T = screen_tables(W16_host, d, L);
+      unsigned char* w = static_cast<unsigned char*>(scratch) + 256;
+      const size_t fb = T.frag.size() * sizeof(uint32_t);
+      e = cudaMemcpyAsync(w, T.frag.data(), fb, cudaMemcpyHostToDevice, st);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(w + fb, T.amax.data(), T.amax.size() * sizeof(float), cudaMemcpyHostToDevice, st);
+      // the tables are host vectors of this call: their copies have to be done before it ends
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e != cudaSuccess) return e;
+      a.frag = reinterpret_cast<const uint4*>(w);
+      a.amax = reinterpret_cast<const float*>(w + fb);
+      a.ksteps = (d / L + 15) / 16;
+      const size_t warps = screen_warp_bytes(d / L) * kScreenWarps;
+      const bool fs = fb + warps <= (size_t)220 * 1024;
+      const size_t smem = warps + (fs ? fb : 0);
+      const int grid = edges_grid(n);
+      if (perm) return fs ? launch_screened<true, true>(a, grid, smem, st) : launch_screened<true, false>(a, grid, smem, st);
+      return fs ? launch_screened<false, true>(a, grid, smem, st) : launch_screened<false, false>(a, grid, smem, st);
+    }
     a.blocks = reinterpret_cast<float2*>(static_cast<unsigned char*>(scratch) + 256);
     return launch_tile_any<true>(a, edges_grid(n), st);
   }

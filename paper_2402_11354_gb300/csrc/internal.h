@@ -61,13 +61,13 @@ peos_status cuda_error(cudaError_t e, const char* what);
 void projections_host(uint64_t seed, int d, int L, int m, float* A, float* B);
 
 // launchers (build.cu).  W16: the vectors k-major with 16 per coordinate (zero padded), read
-// for m <= codes_padded_vecs(); scratch: build_codes_scratch_bytes() bytes, 256-byte aligned
+// for m <= codes_padded_vecs() (W16_host: the same in host memory); scratch: build_codes_scratch_bytes() bytes, 256-byte aligned
 int codes_padded_vecs();
-size_t build_codes_scratch_bytes(int64_t n, int L, int m);
+size_t build_codes_scratch_bytes(int64_t n, int d, int L, int m);
 cudaError_t launch_build_codes(const float* X, int64_t n, int d, const int32_t* nbrs, int R, int L, int m,
-                               const float* A, const float* B, const float* W16, const int32_t* perm,
-                               const float* node_proj, int proj_stride, uint8_t* rec, size_t rec_stride,
-                               void* scratch, cudaStream_t st);
+                               const float* A, const float* B, const float* W16, const float* W16_host,
+                               const int32_t* perm, const float* node_proj, int proj_stride, uint8_t* rec,
+                               size_t rec_stride, void* scratch, cudaStream_t st);
 // projection tables and squared norms of every row
 cudaError_t launch_node_proj(const float* X, int64_t n, int d, int L, int m, const float* A, const float* B,
                              const float* W16, const int32_t* perm, float* out, int out_stride, float* norms,
