@@ -400,6 +400,7 @@ __device__ __forceinline__ void clear(float (&acc)[E][kVecs]) {
 // block of d/L dims, then the partials).
 template <int KU, bool PERM, bool WSMEM>
 __global__ void __launch_bounds__(kTileWarps * 32, 1) node_rows_kernel(TileArgs a) {
+  const int warps = blockDim.x >> 5;  // kTileWarps, fewer where the rows make less than that per SM
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* s_w = reinterpret_cast<float4*>(smem_raw);
   const float4* w = tile_vectors<WSMEM>(a, s_w);
@@ -407,7 +408,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) node_rows_kernel(TileArgs 
   float4* s_e = s_w + (WSMEM ? 2 * a.d * (kVecs / 4) : 0) + (size_t)warp * kRowTile * kTilePitch;
   const int d = a.d, L = a.L, m = a.m, dp = d / L;
   const long long tiles = (a.n + kRowTile - 1) / kRowTile;
-  for (long long t = (long long)blockIdx.x * kTileWarps + warp; t < tiles; t += (long long)gridDim.x * kTileWarps) {
+  for (long long t = (long long)blockIdx.x * warps + warp; t < tiles; t += (long long)gridDim.x * warps) {
     const long long v0 = t * kRowTile;
     auto stage = [&](int c0, int c4) {
       __syncwarp();
@@ -832,6 +833,24 @@ __device__ __forceinline__ int lanes_argmax(float p) {
   return best | ((pv >= 0.0f) ? 0 : 1 << 16);
 }
 
+// sum_k w[16 k] x[k] in order, n a multiple of 4; 16 vector elements in flight
+__device__ __forceinline__ float ordered_sum(const float* w, const float* x, int n) {
+  float p = 0.0f;
+  int k = 0;
+  for (; k + 16 <= n; k += 16) {
+    float v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q] = __ldg(w + (size_t)(k + q) * kVecs);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) p = p + v[q] * x[k + q];
+  }
+  for (; k < n; k += 4) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) p = p + __ldg(w + (size_t)(k + q) * kVecs) * x[k + q];
+  }
+  return p;
+}
+
 template <bool PERM, bool FSMEM>
 __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_kernel(TileArgs a, float c_a, float c_b,
                                                                                    float c_fp) {
@@ -878,7 +897,8 @@ __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_ker
     const float* tv = a.node_proj + (size_t)v * a.proj_stride;
 
     float tot2 = 0.0f, sum = 0.0f, h1 = 0.0f, pending = 0.0f;
-    uint64_t word = 0;
+    bool pending_neg = false;
+    uint64_t word = 0, word0 = 0;
     int wk = 1, wi = 0;
     float S1[4][4], S2[4][4];  // [row of the quad][value]: sum_i P_i and sum_i P_i / ||e_i||
 #pragma unroll
@@ -895,11 +915,30 @@ __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_ker
         // 32 rows of cw4 pieces, a piece per lane and step
         const int dr = 32 / cw4, dc = 32 - dr * cw4;
         int e = lane / cw4, col = lane - e * cw4;
+        if (!PERM) {
+          // the neighbours' pieces all in flight at once, straight into shared memory; v's
+          // few rows are subtracted when they have arrived (each lane its own pieces)
+          int e1 = e, col1 = col;
+          for (int j = 0; j < cw4; ++j) {
+            if (e1 < cnt)
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                               (uint32_t)__cvta_generic_to_shared(s_e + e1 * pitch + col1)),
+                           "l"(a.X + (size_t)queue.u[e1] * d + c0 + 4 * col1)
+                           : "memory");
+            e1 += dr;
+            col1 += dc;
+            if (col1 >= cw4) {
+              col1 -= cw4;
+              ++e1;
+            }
+          }
+          asm volatile("cp.async.wait_all;" ::: "memory");
+        }
 #pragma unroll 4
         for (int j = 0; j < cw4; ++j) {
           if (e < cnt) {
-            const float4 x = row4<PERM>(a.X, queue.u[e], d, c0 + 4 * col, a.perm);
             const float4 y = row4<PERM>(a.X, queue.v[e], d, c0 + 4 * col, a.perm);
+            const float4 x = PERM ? row4<PERM>(a.X, queue.u[e], d, c0 + 4 * col, a.perm) : s_e[e * pitch + col];
             s_e[e * pitch + col] = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
           }
           e += dr;
@@ -913,6 +952,14 @@ __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_ker
       __syncwarp();
 #pragma unroll 1
       for (int b0 = 0; b0 < cw4 * 4; b0 += dp, ++i) {
+        // the block's bound and, from global memory, the first step's vectors, ahead of their use
+        const uint4* f = frag + ((size_t)i * KS * 4) * 32 + lane;
+        const float am = __ldg(a.amax + i);
+        uint4 w[4];
+        if (!FSMEM) {
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt) w[nt] = __ldg(f + nt * 32);
+        }
         // block norm of the lane's own edge, in order
         float n2 = 0.0f;
         uint32_t any = 0;
@@ -955,17 +1002,24 @@ __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_ker
               lo[mt][h] = xl[0];
               lo[mt][2 + h] = xl[1];
             }
-          const uint4* f = frag + ((size_t)(i * KS + ks) * 4) * 32 + lane;
+          uint4 next[4];
+          if (!FSMEM) {
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+              next[nt] = ks + 1 < KS ? __ldg(f + (4 + nt) * 32) : make_uint4(0u, 0u, 0u, 0u);
+          }
 #pragma unroll
           for (int nt = 0; nt < 4; ++nt) {
-            const uint4 w = FSMEM ? f[nt * 32] : __ldg(f + nt * 32);
+            if (FSMEM) w[nt] = f[nt * 32];
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
-              mma_bf16(c[mt][nt], hi[mt], w.x, w.y);
-              mma_bf16(c[mt][nt], lo[mt], w.x, w.y);
-              mma_bf16(c[mt][nt], hi[mt], w.z, w.w);
+              mma_bf16(c[mt][nt], hi[mt], w[nt].x, w[nt].y);
+              mma_bf16(c[mt][nt], lo[mt], w[nt].x, w[nt].y);
+              mma_bf16(c[mt][nt], hi[mt], w[nt].z, w[nt].w);
             }
+            if (!FSMEM) w[nt] = next[nt];
           }
+          f += 4 * 32;
         }
         // row q = 2 mt + h of the quad: columns 2t, 2t + 1 of n-tiles 0, 1 (a) and 2, 3 (b)
         float pa[4][4];
@@ -983,34 +1037,35 @@ __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_ker
         }
         const Top2 top = quad_top2(pa, t);
         int sel = zero ? 0 : top_code(top);
-        const bool open = have && !zero && (small || !top_settled(top, c_a * __ldg(a.amax + i) * bn));
+        const bool open = have && !zero && (small || !top_settled(top, c_a * am * bn));
         for (unsigned todo = __ballot_sync(kFull, open); todo; todo &= todo - 1) {
           const int e = __ffs(todo) - 1;
           float p = 0.0f;
           if (lane < kVecs) {
-            const float* w = a.W + (size_t)(d + i * dp) * kVecs + lane;
-            for (int k = 0; k < dp; ++k) p = p + __ldg(w + (size_t)k * kVecs) * rows[(size_t)e * pitch * 4 + b0 + k];
+            p = ordered_sum(a.W + (size_t)(d + i * dp) * kVecs + lane, rows + (size_t)e * pitch * 4 + b0, dp);
           }
           const int got = lanes_argmax(p);
           if (lane == e) sel = got;
         }
         // the code; its table entry is added a block later, when it has arrived
-        h1 = h1 + pending;
-        if (have) {
-          const float val = __ldg(tv + (i + 1) * m + (sel & 0xffff));
-          pending = (sel >> 16) ? -val : val;
-          word |= ((uint64_t)(sel & 0xffff) | ((uint64_t)(sel >> 16) << (a.bits - 1))) << (wk * a.bits);
-          if (++wk == a.cpw) {
-            cwords[(size_t)wi * R] = word;
-            word = 0;
-            wk = 0;
-            ++wi;
-          }
+        h1 = h1 + (pending_neg ? -pending : pending);
+        pending = __ldg(tv + (i + 1) * m + (sel & 0xffff));
+        pending_neg = (sel >> 16) != 0;
+        word |= ((uint64_t)(sel & 0xffff) | ((uint64_t)(sel >> 16) << (a.bits - 1))) << (wk * a.bits);
+        if (++wk == a.cpw) {
+          if (wi == 0) word0 = word;
+          else if (have) cwords[(size_t)wi * R] = word;
+          word = 0;
+          wk = 0;
+          ++wi;
         }
       }
     }
-    h1 = h1 + pending;
-    if (have && wk > 0) cwords[(size_t)wi * R] = word;
+    h1 = h1 + (pending_neg ? -pending : pending);
+    if (wk > 0) {
+      if (wi == 0) word0 = word;
+      else if (have) cwords[(size_t)wi * R] = word;
+    }
     const float norm = sqrtf(tot2);
     float wr = 1.0f, cr = 0.0f, mean = 0.0f;
     if (norm != 0.0f) {
@@ -1051,16 +1106,9 @@ __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_ker
         s_coef[i] = (b > 0.0f) ? (1.0f - em / b) : 0.0f;
       }
       __syncwarp();
-      float p = 0.0f;
-      if (lane < kVecs) {
-        const float* w = a.W + lane;
-        for (int i = 0; i < L; ++i) {
-          const float cf = s_coef[i];
-#pragma unroll 4
-          for (int k = i * dp; k < (i + 1) * dp; ++k) p = p + __ldg(w + (size_t)k * kVecs) * (lin[k] * cf);
-        }
-      }
-      const int got = lanes_argmax(p);
+      for (int k = lane; k < d; k += 32) lin[k] = lin[k] * s_coef[k / dp];
+      __syncwarp();
+      const int got = lanes_argmax(lane < kVecs ? ordered_sum(a.W + lane, lin, d) : 0.0f);
       if (lane == e) sel0 = got;
     }
     if (have) {
@@ -1068,12 +1116,13 @@ __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_ker
         sel0 = 0;
         h1 = 0.0f;
         for (int i = 0; i < L; ++i) h1 = h1 + __ldg(tv + (i + 1) * m);
-        for (int k = 0; k < a.nwords; ++k) cwords[(size_t)k * R] = 0;
+        word0 = 0;
+        for (int k = 1; k < a.nwords; ++k) cwords[(size_t)k * R] = 0;
       }
       const float v0f = __ldg(tv + (sel0 & 0xffff));
       const float h2 = (sel0 >> 16) ? -v0f : v0f;
       reinterpret_cast<float4*>(rec)[slot] = make_float4(norm, wr, cr, wr * h1 + cr * h2);
-      cwords[0] = cwords[0] | (uint64_t)(sel0 & 0xffff) | ((uint64_t)(sel0 >> 16) << (a.bits - 1));
+      cwords[0] = word0 | (uint64_t)(sel0 & 0xffff) | ((uint64_t)(sel0 >> 16) << (a.bits - 1));
     }
     queue.drop(cnt, lane);
   }
@@ -1211,29 +1260,29 @@ namespace {
 // The tiled kernels' variant for the block length: 4, 2 or 1 coordinates per step, rows
 // read through a permutation or not, the vectors in shared memory or not.
 template <bool EDGES, int KU, bool PERM, bool WSMEM>
-cudaError_t launch_tile(const TileArgs& a, int grid, cudaStream_t st) {
+cudaError_t launch_tile(const TileArgs& a, int grid, int warps, cudaStream_t st) {
   const void* fn = EDGES ? (const void*)build_edges_kernel<KU, PERM, WSMEM> : (const void*)node_rows_kernel<KU, PERM, WSMEM>;
   const size_t per_warp = EDGES ? (size_t)kEdgeTile * kTilePitch * 16 + (size_t)(kEdgeTile + 32) * 12
                                 : (size_t)kRowTile * kTilePitch * 16;
-  const size_t smem = (WSMEM ? (size_t)2 * a.d * kVecs * sizeof(float) : 0) + per_warp * kTileWarps;
+  const size_t smem = (WSMEM ? (size_t)2 * a.d * kVecs * sizeof(float) : 0) + per_warp * warps;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   TileArgs copy = a;
   void* args[] = {&copy};
-  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kTileWarps * 32), args, smem, st);
+  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(warps * 32), args, smem, st);
 }
 template <bool EDGES, int KU>
-cudaError_t launch_tile_ku(const TileArgs& a, int grid, cudaStream_t st) {
+cudaError_t launch_tile_ku(const TileArgs& a, int grid, int warps, cudaStream_t st) {
   const bool ws = a.d <= kMaxSmemVecDim;
-  if (a.perm) return ws ? launch_tile<EDGES, KU, true, true>(a, grid, st) : launch_tile<EDGES, KU, true, false>(a, grid, st);
-  return ws ? launch_tile<EDGES, KU, false, true>(a, grid, st) : launch_tile<EDGES, KU, false, false>(a, grid, st);
+  if (a.perm) return ws ? launch_tile<EDGES, KU, true, true>(a, grid, warps, st) : launch_tile<EDGES, KU, true, false>(a, grid, warps, st);
+  return ws ? launch_tile<EDGES, KU, false, true>(a, grid, warps, st) : launch_tile<EDGES, KU, false, false>(a, grid, warps, st);
 }
 template <bool EDGES>
-cudaError_t launch_tile_any(const TileArgs& a, int grid, cudaStream_t st) {
+cudaError_t launch_tile_any(const TileArgs& a, int grid, int warps, cudaStream_t st) {
   const int dp = a.d / a.L;
-  return dp % 4 == 0   ? launch_tile_ku<EDGES, 4>(a, grid, st)
-         : dp % 2 == 0 ? launch_tile_ku<EDGES, 2>(a, grid, st)
-                       : launch_tile_ku<EDGES, 1>(a, grid, st);
+  return dp % 4 == 0   ? launch_tile_ku<EDGES, 4>(a, grid, warps, st)
+         : dp % 2 == 0 ? launch_tile_ku<EDGES, 2>(a, grid, warps, st)
+                       : launch_tile_ku<EDGES, 1>(a, grid, warps, st);
 }
 
 int edges_grid(int64_t n) { return (int)std::min<int64_t>(num_sms(), (n + kNodeChunk - 1) / kNodeChunk); }
@@ -1305,11 +1354,13 @@ cudaError_t launch_screened(const TileArgs& a, int grid, size_t smem, cudaStream
   if (e != cudaSuccess) return e;
   // a value's error relative to ||a|| ||e_i||: three products of two-term BF16 factors (dropped
   // and rounded terms 3.05 2^-16), their FP32 accumulation (2^-23 per product), and the
-  // sequential sum it stands for (2^-24 per coordinate, with the norms' own rounding)
+  // sequential sum it stands for (2^-24 per coordinate, with the norms' own rounding); for
+  // e_res the same relative to spread (d coordinates), and relative to sum ||e_i|| the
+  // rounding of the two running sums and of the coefficients, (2 L + 8) 2^-24, times 1.5
   const int dp = a.d / a.L;
   const double c = 3.05 * 0x1p-16 + 48.0 * a.ksteps * 0x1p-23 + (2.0 * dp + 8.0) * 0x1p-24;
-  const double fp = (a.d + 2.0 * a.L + 16.0) * 0x1p-23;
-  fn<<<(unsigned)grid, kScreenWarps * 32, smem, st>>>(a, (float)(c * 1.01), (float)(c * 1.01), (float)fp);
+  const double c_res = c + (a.d + 4.0) * 0x1p-24, fp = 1.5 * (2.0 * a.L + 8.0) * 0x1p-24;
+  fn<<<(unsigned)grid, kScreenWarps * 32, smem, st>>>(a, (float)(c * 1.01), (float)(c_res * 1.01), (float)fp);
   return cudaGetLastError();
 }
 
@@ -1370,7 +1421,7 @@ cudaError_t launch_build_codes(const float* X, int64_t n, int d, const int32_t* 
       return fs ? launch_screened<false, true>(a, grid, smem, st) : launch_screened<false, false>(a, grid, smem, st);
     }
     a.blocks = reinterpret_cast<float2*>(static_cast<unsigned char*>(scratch) + 256);
-    return launch_tile_any<true>(a, edges_grid(n), st);
+    return launch_tile_any<true>(a, edges_grid(n), kTileWarps, st);
   }
   const size_t smem = sizeof(float) * ((size_t)R * d + 2 * (size_t)R * L + 4 * (size_t)R +
                                        (size_t)R * (L + 1) * m) +
@@ -1405,8 +1456,9 @@ cudaError_t launch_node_proj(const float* X, int64_t n, int d, int L, int m, con
     a.node_proj = out;
     a.proj_stride = out_stride;
     a.norms = perm ? nullptr : norms;  // the norm sums the stored order of the coordinates
-    const int64_t ctas = (n + (int64_t)kRowTile * kTileWarps - 1) / ((int64_t)kRowTile * kTileWarps);
-    cudaError_t e = launch_tile_any<false>(a, (int)std::min<int64_t>(num_sms(), ctas), st);
+    const int64_t tiles = (n + kRowTile - 1) / kRowTile, sms = num_sms();
+    const int warps = (int)std::min<int64_t>(kTileWarps, (tiles + sms - 1) / sms);
+    cudaError_t e = launch_tile_any<false>(a, (int)std::min<int64_t>(sms, (tiles + warps - 1) / warps), warps, st);
     if (e != cudaSuccess || !perm) return e;
     return launch_row_norms(X, n, d, norms, st);
   }
