@@ -6,10 +6,12 @@
 // is a plain sequential FP32 sum (compiled with --fmad=false), one thread per output,
 // so the results are reproducible bit for bit.
 //
-// Two forms.  Up to 16 vectors per block (m <= 16, every configuration's m) the tiled
+// Three forms.  Up to 16 vectors per block (m <= 16, every configuration's m) the tiled
 // kernels: a thread takes whole edges (or rows) and all 16 sums of each, so that a vector
-// element read from shared memory serves several edges.  For larger m one CTA per node
-// with a thread per sum (node_proj_kernel, build_codes_kernel).
+// element read from shared memory serves several edges.  Where the blocks have 8..64
+// coordinates, a multiple of 4, the edges take the screened form instead: estimates of the
+// sums on the tensor cores settle most codes.  For larger m one CTA per node with a thread
+// per sum (node_proj_kernel, build_codes_kernel).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -247,16 +249,16 @@ __global__ void row_norms_kernel(const float* __restrict__ X, long long n, int d
 // there.  Here a lane owns two edges and keeps the 16 sums of each in registers: per
 // coordinate the warp reads 64 bytes of vectors (one broadcast) and one coordinate of each
 // edge.  A warp walks its nodes' slots, keeps the valid edges in a queue and works on full
-// tiles of 64, so empty slots cost nothing (13.6 of 32 slots are edges).  Measured: index
-// build of 1M x 128 269 -> 10.6 ms, of 50,000 x 960 (L = 24) 106 -> 5.7 ms.  Issue slots are
+// tiles of 64, so empty slots cost nothing (13.6 of 32 slots are edges).  Measured in this
+// form: index build of 1M x 128 269 -> 10.6 ms, of 50,000 x 960 (L = 24) 106 -> 5.7 ms (the
+// screened form below takes both further).  Issue slots are
 // then 57% busy and the rest waits on the rows' gathers: 16 warps 10.4 ms, 20 warps 9.4, 24
 // warps 9.3 (and slower at d = 960); four edges per lane 12.5, coordinates of the next chunk
 // kept in registers 10.8 (one build alone, before its index is freed).
 constexpr int kTileWarps = 20;     // one CTA per SM
 constexpr int kEdgesPerLane = 2;
 constexpr int kEdgeTile = 32 * kEdgesPerLane;
-constexpr int kRowsPerLane = 2;    // node tables
-constexpr int kRowTile = 32 * kRowsPerLane;
+constexpr int kRowsPerLane = 2;    // node tables: rows per lane, one where two leave warps without rows
 constexpr int kTileDims = 16;      // coordinates staged at a time
 // row pitch of the staged tile in 16-byte units: odd, so that lanes reading 16 bytes of 32
 // consecutive rows meet no bank conflict
@@ -395,11 +397,12 @@ __device__ __forceinline__ void clear(float (&acc)[E][kVecs]) {
     for (int j = 0; j < kVecs; ++j) acc[r][j] = 0.0f;
 }
 
-// Projection table of every row, out[v][c][j], and ||v||^2: a warp takes 64 rows, two per
+// Projection table of every row, out[v][c][j], and ||v||^2: a warp takes 32 ROWS rows, ROWS per
 // lane; first the a^i (one sum per block), then the b_j (block by block: a partial sum per
 // block of d/L dims, then the partials).
-template <int KU, bool PERM, bool WSMEM>
+template <int ROWS, int KU, bool PERM, bool WSMEM>
 __global__ void __launch_bounds__(kTileWarps * 32, 1) node_rows_kernel(TileArgs a) {
+  constexpr int kRowTile = 32 * ROWS;
   const int warps = blockDim.x >> 5;  // kTileWarps, fewer where the rows make less than that per SM
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* s_w = reinterpret_cast<float4*>(smem_raw);
@@ -433,16 +436,16 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) node_rows_kernel(TileArgs 
           if (j < m) o[j] = p[j];
       }
     };
-    float acc[kRowsPerLane][kVecs];
-    float nrm[kRowsPerLane];
+    float acc[ROWS][kVecs];
+    float nrm[ROWS];
 #pragma unroll
-    for (int r = 0; r < kRowsPerLane; ++r) nrm[r] = 0.0f;
+    for (int r = 0; r < ROWS; ++r) nrm[r] = 0.0f;
     clear(acc);
     int kk = 0, c = 1;
     for (int c0 = 0; c0 < d; c0 += kTileDims) {
       const int cw = min(kTileDims, d - c0);
       stage(c0, cw >> 2);
-      tile_walk<kRowsPerLane, KU, WSMEM>(
+      tile_walk<ROWS, KU, WSMEM>(
           s_e, w + (size_t)(d + c0) * (kVecs / 4), cw, dp, kk, lane, acc,
           [&](int r, float x) {
             nrm[r] = nrm[r] + x * x;
@@ -450,33 +453,33 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) node_rows_kernel(TileArgs 
           },
           [&] {
 #pragma unroll
-            for (int r = 0; r < kRowsPerLane; ++r) store(r, c, acc[r]);
+            for (int r = 0; r < ROWS; ++r) store(r, c, acc[r]);
             clear(acc);
             ++c;
           });
     }
     if (a.norms) {
 #pragma unroll
-      for (int r = 0; r < kRowsPerLane; ++r)
+      for (int r = 0; r < ROWS; ++r)
         if (v0 + r * 32 + lane < a.n) a.norms[v0 + r * 32 + lane] = nrm[r];
     }
-    float tot[kRowsPerLane][kVecs];
+    float tot[ROWS][kVecs];
     clear(tot);
     for (int c0 = 0; c0 < d; c0 += kTileDims) {
       const int cw = min(kTileDims, d - c0);
       stage(c0, cw >> 2);
-      tile_walk<kRowsPerLane, KU, WSMEM>(
+      tile_walk<ROWS, KU, WSMEM>(
           s_e, w + (size_t)c0 * (kVecs / 4), cw, dp, kk, lane, acc, [&](int, float x) { return x; },
           [&] {
 #pragma unroll
-            for (int r = 0; r < kRowsPerLane; ++r)
+            for (int r = 0; r < ROWS; ++r)
 #pragma unroll
               for (int j = 0; j < kVecs; ++j) tot[r][j] = tot[r][j] + acc[r][j];
             clear(acc);
           });
     }
 #pragma unroll
-    for (int r = 0; r < kRowsPerLane; ++r) {
+    for (int r = 0; r < ROWS; ++r) {
       store(r, 0, tot[r]);
       const long long v = v0 + r * 32 + lane;
       if (v < a.n)
@@ -745,6 +748,13 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) build_edges_kernel(TileArg
 // error bound of both the estimate and the sequential FP32 sum, the 16 sums are formed again
 // in that order and decide, so the codes are those of the tiled form bit for bit.  The block
 // norms are sequential FP32 sums as there (a lane per edge).
+//
+// What bounds it: per tile of 32 edges about 7,000 warp instructions and the rows' gathers;
+// at 16 warps per SM (128 registers: 32 of them the two running sums) 51% of the issue slots
+// are busy.  Rows come by asynchronous copies (1M x 128: plain loads 7.9 ms for the whole
+// build, copies 7.3; 20 warps 8.6), and the sums formed in order keep 16 vector elements in
+// flight (7.3 -> 7.0; 50,000 x 960: 5.1 -> 3.6 ms, where they had been a third of the time).
+// Whole build, tiled form against this one: 1M x 128 10.6 -> 7.0 ms, 50,000 x 960 5.7 -> 3.6.
 constexpr int kScreenWarps = 16;  // one CTA per SM
 constexpr int kScreenDims = 64;   // coordinates staged at a time: whole blocks, at most this many
 constexpr int kMaxCoef = 96;      // blocks per edge (L <= 95, see kMaxCodeWords)
@@ -1259,11 +1269,18 @@ namespace {
 
 // The tiled kernels' variant for the block length: 4, 2 or 1 coordinates per step, rows
 // read through a permutation or not, the vectors in shared memory or not.
-template <bool EDGES, int KU, bool PERM, bool WSMEM>
+// ROWS = 0: the edge kernel, else the row kernel with that many rows per lane.
+template <int ROWS, int KU, bool PERM, bool WSMEM>
 cudaError_t launch_tile(const TileArgs& a, int grid, int warps, cudaStream_t st) {
-  const void* fn = EDGES ? (const void*)build_edges_kernel<KU, PERM, WSMEM> : (const void*)node_rows_kernel<KU, PERM, WSMEM>;
-  const size_t per_warp = EDGES ? (size_t)kEdgeTile * kTilePitch * 16 + (size_t)(kEdgeTile + 32) * 12
-                                : (size_t)kRowTile * kTilePitch * 16;
+  const void* fn;
+  size_t per_warp;
+  if constexpr (ROWS == 0) {
+    fn = (const void*)build_edges_kernel<KU, PERM, WSMEM>;
+    per_warp = (size_t)kEdgeTile * kTilePitch * 16 + (size_t)(kEdgeTile + 32) * 12;
+  } else {
+    fn = (const void*)node_rows_kernel<ROWS, KU, PERM, WSMEM>;
+    per_warp = (size_t)32 * ROWS * kTilePitch * 16;
+  }
   const size_t smem = (WSMEM ? (size_t)2 * a.d * kVecs * sizeof(float) : 0) + per_warp * warps;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1271,22 +1288,25 @@ cudaError_t launch_tile(const TileArgs& a, int grid, int warps, cudaStream_t st)
   void* args[] = {&copy};
   return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(warps * 32), args, smem, st);
 }
-template <bool EDGES, int KU>
+template <int ROWS, int KU>
 cudaError_t launch_tile_ku(const TileArgs& a, int grid, int warps, cudaStream_t st) {
   const bool ws = a.d <= kMaxSmemVecDim;
-  if (a.perm) return ws ? launch_tile<EDGES, KU, true, true>(a, grid, warps, st) : launch_tile<EDGES, KU, true, false>(a, grid, warps, st);
-  return ws ? launch_tile<EDGES, KU, false, true>(a, grid, warps, st) : launch_tile<EDGES, KU, false, false>(a, grid, warps, st);
+  if (a.perm) return ws ? launch_tile<ROWS, KU, true, true>(a, grid, warps, st) : launch_tile<ROWS, KU, true, false>(a, grid, warps, st);
+  return ws ? launch_tile<ROWS, KU, false, true>(a, grid, warps, st) : launch_tile<ROWS, KU, false, false>(a, grid, warps, st);
 }
-template <bool EDGES>
+template <int ROWS>
 cudaError_t launch_tile_any(const TileArgs& a, int grid, int warps, cudaStream_t st) {
   const int dp = a.d / a.L;
-  return dp % 4 == 0   ? launch_tile_ku<EDGES, 4>(a, grid, warps, st)
-         : dp % 2 == 0 ? launch_tile_ku<EDGES, 2>(a, grid, warps, st)
-                       : launch_tile_ku<EDGES, 1>(a, grid, warps, st);
+  return dp % 4 == 0   ? launch_tile_ku<ROWS, 4>(a, grid, warps, st)
+         : dp % 2 == 0 ? launch_tile_ku<ROWS, 2>(a, grid, warps, st)
+                       : launch_tile_ku<ROWS, 1>(a, grid, warps, st);
 }
 
 int edges_grid(int64_t n) { return (int)std::min<int64_t>(num_sms(), (n + kNodeChunk - 1) / kNodeChunk); }
 
+// The shapes of the screened form: a lane's four coordinates of a step lie in one block and
+// start on 16 bytes (blocks a multiple of 4), a step of 16 is at least half full, and whole
+// blocks fit the 64 staged coordinates.  Others take the tiled form.
 bool screened(int d, int L, int m) {
   const int dp = d / L;
   return m <= kVecs && dp % 4 == 0 && dp >= 8 && dp <= kScreenDims && L < kMaxCoef && 32 * screen_pitch(dp) * 4 >= d;
@@ -1421,7 +1441,7 @@ cudaError_t launch_build_codes(const float* X, int64_t n, int d, const int32_t* 
       return fs ? launch_screened<false, true>(a, grid, smem, st) : launch_screened<false, false>(a, grid, smem, st);
     }
     a.blocks = reinterpret_cast<float2*>(static_cast<unsigned char*>(scratch) + 256);
-    return launch_tile_any<true>(a, edges_grid(n), kTileWarps, st);
+    return launch_tile_any<0>(a, edges_grid(n), kTileWarps, st);
   }
   const size_t smem = sizeof(float) * ((size_t)R * d + 2 * (size_t)R * L + 4 * (size_t)R +
                                        (size_t)R * (L + 1) * m) +
@@ -1456,9 +1476,12 @@ cudaError_t launch_node_proj(const float* X, int64_t n, int d, int L, int m, con
     a.node_proj = out;
     a.proj_stride = out_stride;
     a.norms = perm ? nullptr : norms;  // the norm sums the stored order of the coordinates
-    const int64_t tiles = (n + kRowTile - 1) / kRowTile, sms = num_sms();
+    const int64_t sms = num_sms();
+    const int rows = n >= (int64_t)32 * kRowsPerLane * sms * kTileWarps ? kRowsPerLane : 1;
+    const int64_t tiles = (n + 32 * rows - 1) / (32 * rows);
     const int warps = (int)std::min<int64_t>(kTileWarps, (tiles + sms - 1) / sms);
-    cudaError_t e = launch_tile_any<false>(a, (int)std::min<int64_t>(sms, (tiles + warps - 1) / warps), warps, st);
+    const int grid = (int)std::min<int64_t>(sms, (tiles + warps - 1) / warps);
+    cudaError_t e = rows == 1 ? launch_tile_any<1>(a, grid, warps, st) : launch_tile_any<kRowsPerLane>(a, grid, warps, st);
     if (e != cudaSuccess || !perm) return e;
     return launch_row_norms(X, n, d, norms, st);
   }

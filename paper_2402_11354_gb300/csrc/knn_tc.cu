@@ -169,36 +169,55 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// One warp per row, four elements per lane.  LO: the rounding errors' own BF16 values follow
-// the row's hi terms.  norm2: FP32 squared norms (base rows); xmax: the largest of them, as
-// its bits (a NaN's bits are larger than any number's).
+// A warp takes four rows at a time (their loads in flight together), four elements per lane.
+// LO: the rounding errors' own BF16 values follow the row's hi terms.  norm2: FP32 squared
+// norms (base rows); xmax: the largest of them, as its bits (a NaN's bits are larger than any
+// number's).
 template <bool LO>
 __global__ void convert_bf16_kernel(const float* __restrict__ X, long long n, int d, int pitch,
                                     __nv_bfloat16* __restrict__ out, float* __restrict__ norm2,
                                     unsigned* __restrict__ xmax) {
+  constexpr int kAtOnce = 4;
   const int lane = threadIdx.x & 31;
   const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   const size_t row = (size_t)pitch * (LO ? 2 : 1);
   unsigned most = 0;
-  for (long long r = w0; r < n; r += nw) {
-    float s = 0.0f;
+  for (long long r0 = w0 * kAtOnce; r0 < n; r0 += nw * kAtOnce) {
+    float s[kAtOnce];
+#pragma unroll
+    for (int j = 0; j < kAtOnce; ++j) s[j] = 0.0f;
     for (int k = 4 * lane; k < pitch; k += 128) {
-      const float4 v = k < d ? __ldg(reinterpret_cast<const float4*>(X + (size_t)r * d + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      const uint2 h = make_uint2(bf16_pair(v.x, v.y), bf16_pair(v.z, v.w));
-      *reinterpret_cast<uint2*>(out + (size_t)r * row + k) = h;
-      if (LO) {
-        const float4 f = make_float4(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xffff0000u),
-                                     __uint_as_float(h.y << 16), __uint_as_float(h.y & 0xffff0000u));
-        *reinterpret_cast<uint2*>(out + (size_t)r * row + pitch + k) =
-            make_uint2(bf16_pair(v.x - f.x, v.y - f.y), bf16_pair(v.z - f.z, v.w - f.w));
+      float4 v[kAtOnce];
+#pragma unroll
+      for (int j = 0; j < kAtOnce; ++j)
+        v[j] = (k < d && r0 + j < n) ? __ldg(reinterpret_cast<const float4*>(X + (size_t)(r0 + j) * d + k))
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < kAtOnce; ++j) {
+        if (r0 + j >= n) break;
+        const float4 x = v[j];
+        const uint2 h = make_uint2(bf16_pair(x.x, x.y), bf16_pair(x.z, x.w));
+        __nv_bfloat16* o = out + (size_t)(r0 + j) * row + k;
+        *reinterpret_cast<uint2*>(o) = h;
+        if (LO) {
+          const float4 f = make_float4(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xffff0000u),
+                                       __uint_as_float(h.y << 16), __uint_as_float(h.y & 0xffff0000u));
+          *reinterpret_cast<uint2*>(o + pitch) =
+              make_uint2(bf16_pair(x.x - f.x, x.y - f.y), bf16_pair(x.z - f.z, x.w - f.w));
+        }
+        s[j] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
       }
-      s += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
     }
     if (norm2) {
-      s = warp_sum(s);
-      if (lane == 0) norm2[r] = s;
-      most = max(most, __float_as_uint(s));
+#pragma unroll
+      for (int j = 0; j < kAtOnce; ++j) {
+        const float t = warp_sum(s[j]);
+        if (r0 + j < n) {
+          if (lane == 0) norm2[r0 + j] = t;
+          most = max(most, __float_as_uint(t));
+        }
+      }
     }
   }
   if (norm2 && lane == 0 && most) atomicMax(xmax, most);
@@ -931,13 +950,13 @@ cudaError_t run_tc(const TcPlan& p, const float* X, long long n, int d, const fl
   if (e != cudaSuccess) return e;
   const int cols = p.pitch * (PRECISE ? 2 : 1);
   const int cg = sms * 8;
-  convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (nq + 7) / 8), 256, 0, st>>>(Q, nq, d, p.pitch, qb,
+  convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (nq + 31) / 32), 256, 0, st>>>(Q, nq, d, p.pitch, qb,
                                                                                                nullptr, nullptr);
   CUtensorMap mq;
   if (!make_map(&mq, qb, nq, cols, kTcM)) return cudaErrorNotSupported;
   for (int s = 0; s < p.slabs; ++s) {
     const long long r0 = (long long)s * p.slab_rows, rows = std::min(p.slab_rows, n - r0);
-    convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (rows + 7) / 8), 256, 0, st>>>(
+    convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (rows + 31) / 32), 256, 0, st>>>(
         X + (size_t)r0 * d, rows, d, p.pitch, xb, xnorm, xmax);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
