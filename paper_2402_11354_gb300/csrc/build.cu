@@ -1046,7 +1046,9 @@ __global__ void __launch_bounds__(kScreenWarps * 32, 1) build_edges_screened_ker
           }
         }
         const Top2 top = quad_top2(pa, t);
-        int sel = zero ? 0 : top_code(top);
+        // a lane without an edge (stale rows in s_e) reads code 0: its estimates could name a vector
+        // past m, and node 0's table ends there in an index of one node
+        int sel = have && !zero ? top_code(top) : 0;
         const bool open = have && !zero && (small || !top_settled(top, c_a * am * bn));
         for (unsigned todo = __ballot_sync(kFull, open); todo; todo &= todo - 1) {
           const int e = __ffs(todo) - 1;
