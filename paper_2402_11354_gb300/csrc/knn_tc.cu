@@ -27,8 +27,8 @@
 //
 // The precise form proves its result: a row left out of a full list scored no better than
 // that list's worst, so with the score's error bound its distance is known to be above
-// the k-th found, or the query is handed on to the FFMA kernel (knn.cu).  Non-finite or
-// vanishing norms and a CTA that gave up waiting hand every query on.
+// the k-th found, or the query is handed on to the FFMA kernel (knn.cu).  Norms that vanish
+// or come near FP32's range and a CTA that gave up waiting hand every query on.
 //
 // Every wait on an mbarrier is bounded: after kWaitLimitNs of the global timer (or
 // kMaxPolls polls, whichever comes first) the CTA records an error and stops issuing work
@@ -788,7 +788,9 @@ __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_fina
       a.dists_out[(size_t)q * a.k + j] = key == kNoKey ? INFINITY : key_dist(key);
     }
     if (PRECISE && t == 0) {
-      bool proven = *a.err == 0 && isfinite(xm2) && isfinite(q2) && xm2 >= 1e-24 && (q2 >= 1e-24 || q2 == 0.0);
+      // below 1e37 no score, no BF16 term and no distance overflows (|q.x| <= ||q|| ||x||); a
+      // score that did would have entered no list
+      bool proven = *a.err == 0 && xm2 >= 1e-24 && xm2 < 1e37 && (q2 >= 1e-24 || q2 == 0.0) && q2 < 1e37;
       if (left_out != kNoKey) {
         const uint64_t last = s_key[a.k - 1];
         proven = proven && last != kNoKey &&
