@@ -16,6 +16,8 @@
 //      norm does not change the order) in a max-heap in shared memory.  Scores below the
 //      heap's worst wait in a short per-row buffer; when a row's buffer is nearly full all
 //      rows empty theirs side by side.
+//      Where scores are rounded the plain form closes a list at the end of a slice of the base
+//      too, so that a query keeps as many rows as it takes to absorb misranked ones.
 //   3. finalize: the candidates of every segment sorted by score; those that may be among
 //      the k nearest (score within twice the error bound of the k-th) get their exact FP32
 //      squared distance (sequential over the dimensions), and the k smallest by (dist, id)
@@ -38,6 +40,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <float.h>
+#include <math.h>
 
 #include <algorithm>
 #include <mutex>
@@ -172,17 +175,21 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
 // A warp takes four rows at a time (their loads in flight together), four elements per lane.
 // LO: the rounding errors' own BF16 values follow the row's hi terms.  norm2: FP32 squared
 // norms (base rows); xmax: the largest of them, as its bits (a NaN's bits are larger than any
-// number's).
+// number's).  Without LO: `inexact` is set when a score of these rows may be rounded: an
+// element that is not an integer of at most 256, or a squared norm of 2^24 / 3 or more (below,
+// ||x||^2 + 2 |q.x| and all sums on the way stay under 2^24).
+constexpr float kExactNorm2 = 5.5e6f;
 template <bool LO>
 __global__ void convert_bf16_kernel(const float* __restrict__ X, long long n, int d, int pitch,
                                     __nv_bfloat16* __restrict__ out, float* __restrict__ norm2,
-                                    unsigned* __restrict__ xmax) {
+                                    unsigned* __restrict__ xmax, unsigned* __restrict__ inexact) {
   constexpr int kAtOnce = 4;
   const int lane = threadIdx.x & 31;
   const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   const size_t row = (size_t)pitch * (LO ? 2 : 1);
   unsigned most = 0;
+  bool rounded = false;
   for (long long r0 = w0 * kAtOnce; r0 < n; r0 += nw * kAtOnce) {
     float s[kAtOnce];
 #pragma unroll
@@ -207,37 +214,61 @@ __global__ void convert_bf16_kernel(const float* __restrict__ X, long long n, in
               make_uint2(bf16_pair(x.x - f.x, x.y - f.y), bf16_pair(x.z - f.z, x.w - f.w));
         }
         s[j] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+        if (!LO) {
+          const float top = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w)));
+          // adding 1.5 2^23 rounds to an integer (of small values; larger ones fail the other test)
+          const float e = fabsf(((x.x + 12582912.0f) - 12582912.0f) - x.x) + fabsf(((x.y + 12582912.0f) - 12582912.0f) - x.y) +
+                          fabsf(((x.z + 12582912.0f) - 12582912.0f) - x.z) + fabsf(((x.w + 12582912.0f) - 12582912.0f) - x.w);
+          rounded = rounded || !(e == 0.0f && top <= 256.0f);
+        }
       }
     }
-    if (norm2) {
+    if (norm2 || !LO) {
 #pragma unroll
       for (int j = 0; j < kAtOnce; ++j) {
         const float t = warp_sum(s[j]);
-        if (r0 + j < n) {
+        rounded = rounded || !(t < kExactNorm2);
+        if (norm2 && r0 + j < n) {
           if (lane == 0) norm2[r0 + j] = t;
           most = max(most, __float_as_uint(t));
         }
       }
     }
   }
+  if (!LO && __any_sync(kFull, rounded) && lane == 0) *inexact = 1u;
   if (norm2 && lane == 0 && most) atomicMax(xmax, most);
 }
 
-// The tiles of one launch: qt x bt, handed out in equal contiguous shares to G CTAs.
+// The tiles of one launch: qt x bt, handed out in contiguous shares to G CTAs: equal ones, or
+// (`whole`) equal numbers of slices of a query tile's base rows.  A candidate list covers the
+// part of one share, one query tile and one slice: a segment.
 struct TcShare {
   long long units;  // qt * bt
   int bt, G;
-  __host__ __device__ long long start(int c) const { return units * c / G; }
-  // the CTA whose share holds unit u
+  int st, ns;       // tiles per slice, slices per query tile (st >= bt, 1: not sliced)
+  int whole;
+  __host__ __device__ long long start(int c) const {
+    if (!whole) return units * c / G;
+    const long long s = units / bt * ns * c / G;  // the share's first slice
+    return s / ns * bt + s % ns * st;
+  }
+  // the CTA whose share holds unit u (equal shares)
   __host__ __device__ int cta_of(long long u) const { return (int)(((u + 1) * G - 1) / units); }
-  // most CTAs that share one query tile
+  // the list of the segment of CTA c that ends with unit u, among its query tile's lists: from
+  // one segment to the next the slice, the CTA or both go up
+  __host__ __device__ int list_of(long long u, int c) const {
+    const long long q0 = u / bt * bt;
+    return (int)((u - q0) / st) + (whole ? 0 : c - cta_of(q0));
+  }
+  // most lists of one query tile
   __host__ int max_segments() const {
     int most = 1;
-    for (long long q = 0; q * bt < units; ++q) {
-      const int s = cta_of(q * bt + bt - 1) - cta_of(q * bt) + 1;
-      if (s > most) most = s;
-    }
-    return most;
+    if (!whole)
+      for (long long q = 0; q * bt < units; ++q) {
+        const int s = cta_of(q * bt + bt - 1) - cta_of(q * bt) + 1;
+        if (s > most) most = s;
+      }
+    return most + ns - 1;
   }
 };
 
@@ -251,6 +282,7 @@ struct TcArgs {
   uint32_t row0;     // id of the launch's first base row
   int nseg, seg0;    // segments per query in `out`, and the launch's first
   uint64_t* out;     // [nq][nseg][cand] (ordered(approx) << 32 | id), prefilled with kNoKey
+  const unsigned* inexact;  // 0: no score is rounded, and a list may go on past its slice
   int* err;
 };
 
@@ -598,8 +630,10 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
       for (int j = 0; j < kNorms; ++j) xn[j] = r + 32 * j < a.n ? __ldg(a.xnorm + r + 32 * j) : INFINITY;
     };
     if (u0 < u1) load_norms((int)(u0 % bt));
+    const long long st = PRECISE || __ldg(a.inexact) == 0u ? bt : a.share.st;
     for (long long u = u0; u < u1;) {
-      const long long qt = u / bt, ue = min(u1, (qt + 1) * bt);
+      const long long qt = u / bt, qe = (qt + 1) * bt;
+      const long long ue = min(min(u1, qe), qt * bt + ((u - qt * bt) / st + 1) * st);
       for (int i = half; i < a.cand; i += kHalves) list.heap[(size_t)i * kRows] = kNoKey;
       list.worst_f = FLT_MAX;
       quarter_sync<EW>(quarter);
@@ -609,7 +643,7 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
         const uint32_t id0 = a.row0 + (uint32_t)((u - qt * bt) * kTcN) + half * kCols;
 #pragma unroll
         for (int j = 0; j < kNorms; ++j) my_xn[lane + 32 * j] = xn[j];
-        if (u + 1 < u1) load_norms(u + 1 < ue ? (int)(u + 1 - qt * bt) : 0);
+        if (u + 1 < u1) load_norms(u + 1 < qe ? (int)(u + 1 - qt * bt) : 0);
         if (!mbar_wait(accf + b, (t >> 1) & 1)) s_fail = 1;
         __syncwarp();
         ok = !__any_sync(kFull, s_fail != 0);
@@ -639,7 +673,7 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
       list.flush();
       quarter_sync<EW>(quarter);
       if (ok && qt * kTcM + row < a.nq) {
-        const int seg = a.seg0 + blockIdx.x - a.share.cta_of(qt * bt);
+        const int seg = a.seg0 + a.share.list_of(ue - 1, blockIdx.x);
         uint64_t* o = a.out + ((size_t)(qt * kTcM + row) * a.nseg + seg) * a.cand;
         for (int i = half; i < a.cand; i += kHalves) o[i] = list.heap[(size_t)i * kRows];
       }
@@ -722,7 +756,21 @@ __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_fina
     for (int o = 16; o > 0; o >>= 1) q2 += __shfl_xor_sync(kFull, q2, o);
     const double err = (double)a.c_dot * sqrt(q2) * xm + (double)a.c_norm * xm2;
     const uint64_t* src = a.cand + (size_t)q * ncand;
-    for (int i = t; i < a.P; i += WPQ * 32) s_key[i] = i < ncand ? src[i] : kNoKey;
+    int P = a.P;
+    if (WPQ == 1) {  // the filled slots alone
+      int have = 0;
+      for (int i0 = 0; i0 < ncand; i0 += 32) {
+        const uint64_t key = i0 + lane < ncand ? src[i0 + lane] : kNoKey;
+        const unsigned m = __ballot_sync(kFull, key != kNoKey);
+        if (key != kNoKey) s_key[have + __popc(m & ((1u << lane) - 1u))] = key;
+        have += __popc(m);
+      }
+      P = 1;
+      while (P < have || P < a.k) P <<= 1;
+      for (int i = have + lane; i < P; i += 32) s_key[i] = kNoKey;
+    } else {
+      for (int i = t; i < P; i += WPQ * 32) s_key[i] = i < ncand ? src[i] : kNoKey;
+    }
     // the smallest root of a full list: no row left out scored below it
     uint64_t left_out = kNoKey;
     if (PRECISE) {
@@ -731,7 +779,7 @@ __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_fina
       for (int o = 16; o > 0; o >>= 1) left_out = min(left_out, (uint64_t)__shfl_xor_sync(kFull, (unsigned long long)left_out, o));
     }
     group_sync<WPQ>();
-    group_sort<WPQ>(s_key, a.P, t);
+    group_sort<WPQ>(s_key, P, t);
     // a candidate more than two error bounds above the k-th score is farther than k others,
     // also in FP32
     const double fp = (double)(d + 4) * 0x1p-23;
@@ -739,7 +787,7 @@ __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_fina
     const double thr = kth == kNoKey ? INFINITY : (double)key_score(kth) + 2.0 * err + fp * fabs((double)key_score(kth) + err + q2);
     int m = 0;  // candidates to measure: the first m
     {
-      int lo = 0, hi = a.P;
+      int lo = 0, hi = P;
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         const uint64_t key = s_key[mid];
@@ -751,7 +799,7 @@ __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_fina
     while (P2 < m) P2 <<= 1;
     if (P2 < a.k) {
       while (P2 < a.k) P2 <<= 1;
-      P2 = min(P2, a.P);
+      P2 = min(P2, P);
     }
     group_sync<WPQ>();
     for (int i = t; i < P2; i += WPQ * 32) {
@@ -848,20 +896,61 @@ struct TcPlan {
   size_t xb, qb, xnorm, cand_buf, flags, total;  // scratch offsets
 };
 
-TcShare tc_share(long long n, long long nq, int cand, int slabs, int sms) {
+// cost of a list's start in tiles: it takes about cand (1 + ln(rows / cand)) insertions
+double list_tiles(double rows, int cand) { return 64.0 * (rows > cand ? 1.0 + log(rows / cand) : 1.0); }
+
+// The slices of the base whose best `cand` rows a query keeps where scores are rounded (that
+// many lists are what absorbs misranked rows; with the lists of the CTAs' shares alone, as few
+// as one, 6 of 20,000 queries over 1M x 100 unit vectors lost one of their 10 nearest): the
+// number that would be quickest with a CTA per slice and query tile, among slices of at least
+// 4 tiles.
+int tc_slices(long long n, long long qt, int cand, int sms) {
+  const long long most = std::max(1LL, std::min((n + 4LL * kTcN - 1) / (4LL * kTcN), (long long)kMaxCandTotal / cand));
+  long long best = 1;
+  double best_cost = -1.0;
+  for (long long s = 1; s <= most; ++s) {
+    const double rows = (double)((n + s - 1) / s);
+    const double cost = (double)((qt * s + sms - 1) / sms) * (ceil(rows / kTcN) + list_tiles(rows, cand));
+    if (best_cost < 0.0 || cost < best_cost) {
+      best_cost = cost;
+      best = s;
+    }
+  }
+  return (int)best;
+}
+
+TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, int sms) {
   TcShare s;
   const long long qt = (nq + kTcM - 1) / kTcM;
   s.bt = (int)((n + kTcN - 1) / kTcN);
   s.units = qt * s.bt;
+  s.st = s.bt;
+  s.ns = 1;
+  s.whole = 0;
+  if (!precise) {
+    const int want = tc_slices(n, qt, cand, sms);
+    s.st = (int)(((n + want - 1) / want + kTcN - 1) / kTcN);
+    s.ns = (s.bt + s.st - 1) / s.st;
+  }
   // one CTA per SM; no more than kMaxCandTotal candidates per query over its segments (a
   // query tile's share spans at most ceil(G / qt) + 1 CTAs), and segments of at least 4
   // tiles, below which the lists' start-up would outweigh the tiles
   long long G = sms;
   const long long most = kMaxCandTotal / ((long long)cand * slabs);
-  if (most >= 2) G = std::min(G, std::max(1LL, (most - 1) * qt));
+  const long long room = most - s.ns + 1;  // lists of a query tile beside its slices' own
+  if (room >= 2) G = std::min(G, std::max(1LL, (room - 1) * qt));
   else G = std::min(G, qt);
   G = std::min(G, std::max(1LL, s.units / 4));
   s.G = (int)std::max(1LL, G);
+  if (s.ns > 1) {
+    // whole slices where their uneven numbers cost less than the lists cut by equal shares
+    const double start = list_tiles(256.0 * s.st, cand), slices = (double)(qt * s.ns);
+    const int gw = (int)std::min<long long>(sms, qt * s.ns);
+    if (room < 2 || ceil(slices / gw) * (s.st + start) <= (double)s.units / s.G + (slices / s.G + 1.0) * start) {
+      s.whole = 1;
+      s.G = gw;
+    }
+  }
   return s;
 }
 
@@ -883,10 +972,10 @@ bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcP
     p->slabs = (int)((n + fit - 1) / fit);
     p->slab_rows = p->slabs > 1 ? fit : n;
   }
-  p->share = tc_share(p->slab_rows, nq, p->cand, p->slabs, sms);
+  p->share = tc_share(p->slab_rows, nq, p->cand, p->slabs, precise, sms);
   int seg = p->share.max_segments();
   if (p->slabs > 1) {
-    const TcShare last = tc_share(n - (long long)(p->slabs - 1) * p->slab_rows, nq, p->cand, p->slabs, sms);
+    const TcShare last = tc_share(n - (long long)(p->slabs - 1) * p->slab_rows, nq, p->cand, p->slabs, precise, sms);
     seg = std::max(seg, last.max_segments());
   }
   p->nseg = seg * p->slabs;
@@ -900,7 +989,7 @@ bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcP
   o += up256((size_t)p->slab_rows * 4);
   p->cand_buf = o;
   o += up256((size_t)nq * p->nseg * p->cand * 8);
-  p->flags = o;  // xmax, err, left count
+  p->flags = o;  // xmax, inexact, err, left count
   o += kTcPad;
   p->total = o;
   return true;
@@ -948,18 +1037,18 @@ cudaError_t run_tc(const TcPlan& p, const float* X, long long n, int d, const fl
   uint64_t* cand_buf = reinterpret_cast<uint64_t*>(w + p.cand_buf);
   unsigned* xmax = reinterpret_cast<unsigned*>(w + p.flags);
   cudaError_t e = cudaMemsetAsync(cand_buf, 0xff, (size_t)nq * p.nseg * p.cand * 8, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(xmax, 0, sizeof(unsigned), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(xmax, 0, 2 * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   const int cols = p.pitch * (PRECISE ? 2 : 1);
   const int cg = sms * 8;
   convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (nq + 31) / 32), 256, 0, st>>>(Q, nq, d, p.pitch, qb,
-                                                                                               nullptr, nullptr);
+                                                                                               nullptr, nullptr, xmax + 1);
   CUtensorMap mq;
   if (!make_map(&mq, qb, nq, cols, kTcM)) return cudaErrorNotSupported;
   for (int s = 0; s < p.slabs; ++s) {
     const long long r0 = (long long)s * p.slab_rows, rows = std::min(p.slab_rows, n - r0);
     convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (rows + 31) / 32), 256, 0, st>>>(
-        X + (size_t)r0 * d, rows, d, p.pitch, xb, xnorm, xmax);
+        X + (size_t)r0 * d, rows, d, p.pitch, xb, xnorm, xmax, xmax + 1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     CUtensorMap mx;
@@ -968,13 +1057,14 @@ cudaError_t run_tc(const TcPlan& p, const float* X, long long n, int d, const fl
     ta.xnorm = xnorm;
     ta.n = rows;
     ta.nq = nq;
-    ta.share = rows == p.slab_rows ? p.share : tc_share(rows, nq, p.cand, p.slabs, sms);
+    ta.share = rows == p.slab_rows ? p.share : tc_share(rows, nq, p.cand, p.slabs, PRECISE, sms);
     ta.kchunks = p.pitch / kTcK;
     ta.cand = p.cand;
     ta.row0 = (uint32_t)r0;
     ta.nseg = p.nseg;
     ta.seg0 = s * (p.nseg / p.slabs);
     ta.out = cand_buf;
+    ta.inexact = xmax + 1;
     ta.err = err;
     bool fits = false;
     e = launch_tc<PRECISE, true, 8>(mq, mx, ta, maxsm, st, &fits);
@@ -1057,7 +1147,7 @@ cudaError_t launch_knn_exact(const float* X, long long n, int d, const float* Q,
   TcPlan p;
   if (!tc_plan(n, nq, d, k, true, sms, &p)) return cudaErrorInvalidConfiguration;
   unsigned char* w = static_cast<unsigned char*>(scratch);
-  int* err = reinterpret_cast<int*>(w + p.flags) + 1;
+  int* err = reinterpret_cast<int*>(w + p.flags) + 2;
   int* left_count = err + 1;
   int32_t* left = reinterpret_cast<int32_t*>(w + p.total);
   cudaError_t e = cudaMemsetAsync(err, 0, 2 * sizeof(int), st);
