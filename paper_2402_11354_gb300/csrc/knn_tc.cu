@@ -378,7 +378,12 @@ __device__ __forceinline__ void unlock_rows(int* lock, int lane) {
   if (lane == 0) atomicExch(lock, 0);
 }
 
+// ORDERED: one warp per row, so that the columns arrive in order and a score equal to the
+// worst kept one never enters.
+template <bool ORDERED>
 struct RowList {
+  // no score yet: above every finite one, and not passed by +inf (a column past the base)
+  static constexpr float kNoWorst = ORDERED ? INFINITY : FLT_MAX;
   uint64_t* heap;
   uint2* pend;
   int* lock;            // null: one warp per row
@@ -386,6 +391,8 @@ struct RowList {
   int cand;
   int waiting;
   float worst_f;        // the root's score when this warp last saw it (never below the root's now)
+  float below_f;        // the next lower score,
+  uint32_t worst_id;    // and the root's id
 
   // warp-wide
   __device__ __forceinline__ void flush() {
@@ -397,16 +404,22 @@ struct RowList {
     }
     const uint64_t worst = heap_insert(heap, pend, cand, waiting);
     waiting = 0;
-    worst_f = key_score(worst);
+    worst_f = worst == kNoKey ? kNoWorst : key_score(worst);
+    if (!ORDERED) {
+      below_f = worst_f == 0.0f ? -FLT_TRUE_MIN : key_score(worst - (1ull << 32));
+      worst_id = (uint32_t)worst;
+    }
     if (lock) unlock_rows(lock, lane);
   }
 };
 
 // One group of scores of the row: a group whose best is not below any row's worst kept score
 // costs a fused multiply-add and a minimum per column.  A score equal to the worst kept one
-// may still enter by its id (the two halves' columns do not arrive in order): the keys decide.
-template <int kGroup, int kPend>
-__device__ __forceinline__ void screen(const uint32_t (&v)[kGroup], const float* xn, uint32_t id0, RowList& L) {
+// enters by a lower id (the two halves' columns do not arrive in order); on a base of equal
+// rows all others stop here (300,000 x 100, 2,000 queries, k = 10: buffered and refused by
+// their keys they took 2.38 ms against 0.54).
+template <int kGroup, int kPend, bool ORDERED>
+__device__ __forceinline__ void screen(const uint32_t (&v)[kGroup], const float* xn, uint32_t id0, RowList<ORDERED>& L) {
   float sc[kGroup];
 #pragma unroll
   for (int u = 0; u < kGroup; u += 4) {
@@ -420,11 +433,12 @@ __device__ __forceinline__ void screen(const uint32_t (&v)[kGroup], const float*
 #pragma unroll
   for (int u = 1; u + 1 < kGroup; u += 2) best = fminf(best, fminf(sc[u], sc[u + 1]));
   best = fminf(best, sc[kGroup - 1]);
-  if (!__any_sync(kFull, best <= L.worst_f)) return;
+  if (!__any_sync(kFull, ORDERED ? best < L.worst_f : best <= L.worst_f)) return;
   if (__any_sync(kFull, L.waiting > kPend - kGroup)) L.flush();
+  const float most = !ORDERED && id0 > L.worst_id ? L.below_f : L.worst_f;  // equal scores by a lower id only
 #pragma unroll
   for (int u = 0; u < kGroup; ++u) {
-    if (sc[u] <= L.worst_f) {
+    if (ORDERED ? sc[u] < most : sc[u] <= most) {
       L.pend[(size_t)L.waiting * kRows] = make_uint2(__float_as_uint(sc[u]), id0 + (uint32_t)u);
       ++L.waiting;
     }
@@ -616,8 +630,9 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
     // warp of the other half
     const int quarter = warp & 3, half = warp >> 2, row = quarter * 32 + lane;
     constexpr int kCols = kTcN / kHalves;
-    RowList list{keys + row, pend + (size_t)half * kPend * kRows + row, kHalves > 1 ? &s_lock[quarter] : nullptr,
-                 &s_fail, a.cand, 0, FLT_MAX};
+    using List = RowList<kHalves == 1>;
+    List list{keys + row, pend + (size_t)half * kPend * kRows + row, kHalves > 1 ? &s_lock[quarter] : nullptr,
+              &s_fail, a.cand, 0, List::kNoWorst, List::kNoWorst, 0xffffffffu};
     uint32_t t = 0;
     bool ok = true;
     // ||x||^2 of the warp's columns of the next tile, loaded a tile ahead
@@ -635,7 +650,8 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
       const long long qt = u / bt, qe = (qt + 1) * bt;
       const long long ue = min(min(u1, qe), qt * bt + ((u - qt * bt) / st + 1) * st);
       for (int i = half; i < a.cand; i += kHalves) list.heap[(size_t)i * kRows] = kNoKey;
-      list.worst_f = FLT_MAX;
+      list.worst_f = List::kNoWorst;
+      list.worst_id = 0xffffffffu;
       quarter_sync<EW>(quarter);
       // after a failed wait the warp only keeps up with its barriers
       for (; u < ue && ok; ++u, ++t) {
@@ -657,11 +673,11 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
 #pragma unroll 1
         for (int c0 = 0; c0 < kCols; c0 += 2 * kGroup) {
           tmem_ld(vb, taddr + c0 + kGroup);
-          screen<kGroup, kPend>(va, my_xn + c0, id0 + c0, list);
+          screen<kGroup, kPend, kHalves == 1>(va, my_xn + c0, id0 + c0, list);
           __syncwarp();
           tmem_wait(vb);
           if (c0 + 2 * kGroup < kCols) tmem_ld(va, taddr + c0 + 2 * kGroup);
-          screen<kGroup, kPend>(vb, my_xn + c0 + kGroup, id0 + c0 + kGroup, list);
+          screen<kGroup, kPend, kHalves == 1>(vb, my_xn + c0 + kGroup, id0 + c0 + kGroup, list);
           __syncwarp();
           tmem_wait(va);
         }
