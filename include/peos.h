@@ -493,8 +493,8 @@ peos_status peos_selftest_bounded_wait(int64_t limit_us, int32_t* gave_up, void*
  * for each query the k base rows with the smallest squared l2 distance, ascending
  * (dist, id).  Distances are exact FP32 sums of squared differences.
  * base/queries: device PEOS_F32; ids_out [nq][k], dists_out [nq][k] device;
- * 1 <= k <= 256.  Uses library-owned scratch of at most about 1 GiB (the queries run in
- * slices whose per-chunk candidate lists fit in it). */
+ * 1 <= k <= 256.  Uses library-owned scratch of at most about 1 GiB (queries and base run in
+ * slices whose converted rows and candidate lists fit in it). */
 peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* queries, int32_t k,
                                 int32_t* ids_out, float* dists_out, void* stream);
 

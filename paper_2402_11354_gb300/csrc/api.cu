@@ -5,6 +5,7 @@
 #include <math.h>
 #include <stdio.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -1085,8 +1086,9 @@ peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* quer
   if (queries->n > 0 && (!ids_out || !dists_out)) return set_error(PEOS_E_INVAL, "NULL output");
   if (queries->n == 0) return PEOS_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // the per-chunk lists take nq x chunks x k keys: the queries go in slices whose lists
-  // fit in 1 GiB (at least 32 queries, one CTA's worth, per slice)
+  // the FFMA form's per-chunk lists take nq x chunks x k keys: its queries go in slices whose
+  // lists fit in 1 GiB (at least 32 queries, one CTA's worth, per slice).  The scores' queries
+  // go in slices of their own; the lists of the queries they leave over take the same memory.
   const size_t per_query = knn_scratch_bytes(base->n, 1, k);
   int64_t slice = (int64_t)((size_t)1 << 30) / (int64_t)per_query;
   slice = slice < 32 ? 32 : slice - slice % 32;
@@ -1095,30 +1097,40 @@ peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* quer
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  size_t exact = base->n >= kKnnExactMinRows && base->n <= 0x7fffffffLL
-                     ? knn_exact_scratch_bytes(base->n, slice, base->d, k, sms)
-                     : 0;
+  const bool scores = base->n >= kKnnExactMinRows && base->n <= 0x7fffffffLL;
+  int64_t exact = scores ? knn_exact_slice(base->n, queries->n, base->d, k, sms) : 0;
   StreamScratch scratch(s);
-  cudaError_t e = scratch.alloc(lists + exact);
-  if (e == cudaErrorMemoryAllocation && exact) {  // the converted base does not fit: FFMA alone
-    (void)cudaGetLastError();
+  cudaError_t e = cudaErrorMemoryAllocation;
+  if (exact) {
+    size_t bytes = knn_exact_left_bytes(exact) + knn_scratch_bytes(base->n, std::min(slice, exact), k);
+    bytes = std::max(bytes, knn_exact_scratch_bytes(base->n, exact, base->d, k, sms));
+    if (queries->n % exact)
+      bytes = std::max(bytes, knn_exact_scratch_bytes(base->n, queries->n % exact, base->d, k, sms));
+    e = scratch.alloc(bytes);
+    if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();  // the converted base does not fit: FFMA alone
+  }
+  if (e == cudaErrorMemoryAllocation) {
     exact = 0;
     e = scratch.alloc(lists);
   }
   if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync knn scratch");
   const float* X = static_cast<const float*>(base->data);
   const float* Q = static_cast<const float*>(queries->data);
-  void* tc = static_cast<char*>(scratch.p) + lists;
-  for (int64_t q0 = 0; q0 < queries->n; q0 += slice) {
-    const int64_t nq = queries->n - q0 < slice ? queries->n - q0 : slice;
+  const int64_t step = exact ? exact : slice;
+  for (int64_t q0 = 0; q0 < queries->n; q0 += step) {
+    const int64_t nq = std::min(step, queries->n - q0);
+    const float* q = Q + (size_t)q0 * base->d;
     int32_t* ids = ids_out + (size_t)q0 * k;
     float* dists = dists_out + (size_t)q0 * k;
-    const size_t need = exact ? knn_exact_scratch_bytes(base->n, nq, base->d, k, sms) : 0;
     e = cudaErrorNotSupported;
-    if (need > 0 && need <= exact)
-      e = launch_knn_exact(X, base->n, base->d, Q + (size_t)q0 * base->d, nq, k, ids, dists, tc, scratch.p, sms, s);
-    if (e == cudaErrorNotSupported)  // also where tensor maps are not available
-      e = launch_knn(X, base->n, base->d, Q + (size_t)q0 * base->d, nq, k, ids, dists, scratch.p, s);
+    if (exact && knn_exact_scratch_bytes(base->n, nq, base->d, k, sms))
+      e = launch_knn_exact(X, base->n, base->d, q, nq, k, ids, dists, scratch.p, slice, sms, s);
+    if (e == cudaErrorNotSupported) {  // also where tensor maps are not available
+      e = cudaSuccess;
+      for (int64_t o = 0; o < nq && e == cudaSuccess; o += slice)
+        e = launch_knn(X, base->n, base->d, q + (size_t)o * base->d, std::min(slice, nq - o), k, ids + (size_t)o * k,
+                       dists + (size_t)o * k, scratch.p, s);
+    }
     if (e != cudaSuccess) return cuda_error(e, "knn launch");
   }
   return PEOS_OK;

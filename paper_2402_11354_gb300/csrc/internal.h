@@ -177,10 +177,10 @@ cudaError_t launch_edge_stats(const peos_codes_s* c, const float* q, int v, floa
 
 // brute force (knn.cu)
 size_t knn_scratch_bytes(int64_t n, int64_t nq, int k);
-// (qlist, qcount: device memory; only the listed queries, at most nq of them)
+// (qlist, qcount: device memory; only the listed queries from qfirst on, at most nq of them)
 cudaError_t launch_knn(const float* X, int64_t n, int d, const float* Q, int64_t nq, int k, int32_t* ids_out,
                        float* dists_out, void* scratch, cudaStream_t st, const int32_t* qlist = nullptr,
-                       const int* qcount = nullptr);
+                       const int* qcount = nullptr, int64_t qfirst = 0);
 
 // stage tracing (api.cu): while tracing is on, each search records events around its
 // stages (query tables, search kernel, re-rank) on its stream
@@ -195,10 +195,14 @@ void trace_end(const TraceCall& tc);
 int knn_tc_max_k();
 cudaError_t launch_bounded_wait_probe(long long limit_ns, int* gave_up, cudaStream_t st);
 // the same results as launch_knn from two-term BF16 scores, with launch_knn itself for the
-// queries they cannot prove; scratch 0: not served (k too large, or too many candidates)
+// queries they cannot prove (ffma_slice of them at a time, whose lists overlay the scores'
+// scratch, from left_bytes(nq) on).  slice: queries per call whose scratch keeps to about 1 GiB;
+// slice or bytes 0: the scores do not serve (k too large, or too many candidates)
+size_t knn_exact_left_bytes(long long nq);
 size_t knn_exact_scratch_bytes(long long n, long long nq, int d, int k, int sms);
+long long knn_exact_slice(long long n, long long nq, int d, int k, int sms);
 cudaError_t launch_knn_exact(const float* X, long long n, int d, const float* Q, long long nq, int k, int32_t* ids_out,
-                             float* dists_out, void* scratch, void* ffma_scratch, int sms, cudaStream_t st);
+                             float* dists_out, void* scratch, long long ffma_slice, int sms, cudaStream_t st);
 size_t knn_tc_scratch_bytes(long long n, long long nq, int d, int k, int sms);
 cudaError_t launch_knn_tc(const float* X, long long n, int d, const float* Q, long long nq, int k, int32_t* ids_out,
                           float* dists_out, void* scratch, int* err_flag, cudaStream_t st);

@@ -975,7 +975,11 @@ TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, i
 // k, fewer where shared memory ends (a shorter slack only proves fewer queries).
 constexpr int kMaxCand = 113;
 
-// precise: the base is converted in slabs of at most 1 GiB.  False: not served.
+// The precise form's scratch stays within 1 GiB (the bound that peos_knn_bruteforce states):
+// the base is converted in slabs of at most 768 MiB, the rest holds queries and lists.
+constexpr size_t kExactBytes = (size_t)1 << 30, kExactSlabBytes = (size_t)768 << 20;
+
+// False: not served.
 bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcPlan* p) {
   p->pitch = tc_pitch(d);
   p->cand = precise ? std::min(k + 16, kMaxCand) : k + 16;
@@ -984,7 +988,7 @@ bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcP
   p->slab_rows = n;
   p->slabs = 1;
   if (precise) {
-    const long long fit = std::max<long long>(kTcN, (long long)(((size_t)1 << 30) / row) / kTcN * kTcN);
+    const long long fit = std::max<long long>(kTcN, (long long)(kExactSlabBytes / row) / kTcN * kTcN);
     p->slabs = (int)((n + fit - 1) / fit);
     p->slab_rows = p->slabs > 1 ? fit : n;
   }
@@ -1005,7 +1009,7 @@ bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcP
   o += up256((size_t)p->slab_rows * 4);
   p->cand_buf = o;
   o += up256((size_t)nq * p->nseg * p->cand * 8);
-  p->flags = o;  // xmax, inexact, err, left count
+  p->flags = o;  // xmax, inexact
   o += kTcPad;
   p->total = o;
   return true;
@@ -1153,25 +1157,43 @@ cudaError_t launch_knn_tc(const float* X, long long n, int d, const float* Q, lo
 
 // ---- exact brute force: the precise form, and the FFMA kernel for what it leaves -----------
 
+namespace {
+// what has to outlast the scores: the list of queries left over and its length
+size_t left_bytes(long long nq) { return kTcPad + up256((size_t)nq * 4); }
+}  // namespace
+
 size_t knn_exact_scratch_bytes(long long n, long long nq, int d, int k, int sms) {
   TcPlan p;
-  return tc_plan(n, nq, d, k, true, sms, &p) ? p.total + up256((size_t)nq * 4) : 0;
+  return tc_plan(n, nq, d, k, true, sms, &p) ? left_bytes(nq) + p.total : 0;
+}
+
+long long knn_exact_slice(long long n, long long nq, int d, int k, int sms) {
+  for (long long parts = 1;; parts *= 2) {
+    long long slice = (nq + parts - 1) / parts;
+    if (parts > 1) slice = (slice + kTcM - 1) / kTcM * kTcM;
+    const size_t bytes = knn_exact_scratch_bytes(n, slice, d, k, sms);
+    if (!bytes || bytes <= kExactBytes || slice <= kTcM) return bytes ? slice : 0;
+  }
 }
 
 cudaError_t launch_knn_exact(const float* X, long long n, int d, const float* Q, long long nq, int k, int32_t* ids_out,
-                             float* dists_out, void* scratch, void* ffma_scratch, int sms, cudaStream_t st) {
+                             float* dists_out, void* scratch, long long ffma_slice, int sms, cudaStream_t st) {
   TcPlan p;
   if (!tc_plan(n, nq, d, k, true, sms, &p)) return cudaErrorInvalidConfiguration;
-  unsigned char* w = static_cast<unsigned char*>(scratch);
-  int* err = reinterpret_cast<int*>(w + p.flags) + 2;
+  int* err = static_cast<int*>(scratch);
   int* left_count = err + 1;
-  int32_t* left = reinterpret_cast<int32_t*>(w + p.total);
+  int32_t* left = reinterpret_cast<int32_t*>(static_cast<unsigned char*>(scratch) + kTcPad);
+  unsigned char* w = static_cast<unsigned char*>(scratch) + left_bytes(nq);
   cudaError_t e = cudaMemsetAsync(err, 0, 2 * sizeof(int), st);
   if (e != cudaSuccess) return e;
   e = run_tc<true>(p, X, n, d, Q, nq, k, ids_out, dists_out, w, err, left_count, left, sms, st);
-  if (e != cudaSuccess) return e;
-  return launch_knn(X, n, d, Q, nq, k, ids_out, dists_out, ffma_scratch, st, left, left_count);
+  // the scores are done with w when these run; all but the list's own are empty launches
+  for (long long q = 0; q < nq && e == cudaSuccess; q += ffma_slice)
+    e = launch_knn(X, n, d, Q, std::min(ffma_slice, nq - q), k, ids_out, dists_out, w, st, left, left_count, q);
+  return e;
 }
+
+size_t knn_exact_left_bytes(long long nq) { return left_bytes(nq); }
 
 cudaError_t launch_bounded_wait_probe(long long limit_ns, int* gave_up, cudaStream_t st) {
   bounded_wait_probe_kernel<<<1, 32, 0, st>>>(limit_ns, gave_up);
