@@ -1067,10 +1067,10 @@ peos_status peos_selftest_bounded_wait(int64_t limit_us, int32_t* gave_up, void*
   return PEOS_OK;
 }
 
-// Bases from this size on take the tensor-core scores first (d = 100, k = 10, 1 / 2,000
-// queries, FFMA alone against scores: 2,048 rows 199 / 246 us against 114 / 172; 16,384 rows
-// 1187 / 1366 against 123 / 324; 300,000 rows 1.5 / 6.8 ms against 0.25 / 0.94; below, the
-// six launches cost what one does).
+// Bases from this size on take the tensor-core scores first where they are estimated to be
+// quicker (knn_exact_scratch_bytes; d = 100, k = 10, 1 / 2,000 queries, FFMA alone against
+// scores: 2,048 rows 199 / 246 us against 114 / 172; 16,384 rows 1187 / 1366 against 123 / 324;
+// 300,000 rows 1.5 / 6.8 ms against 0.23 / 0.89; below, the six launches cost what one does).
 static constexpr int64_t kKnnExactMinRows = 2048;
 
 peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* queries, int32_t k, int32_t* ids_out,

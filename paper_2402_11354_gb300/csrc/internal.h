@@ -197,7 +197,7 @@ cudaError_t launch_bounded_wait_probe(long long limit_ns, int* gave_up, cudaStre
 // the same results as launch_knn from two-term BF16 scores, with launch_knn itself for the
 // queries they cannot prove (ffma_slice of them at a time, whose lists overlay the scores'
 // scratch, from left_bytes(nq) on).  slice: queries per call whose scratch keeps to about 1 GiB;
-// slice or bytes 0: the scores do not serve (k too large, or too many candidates)
+// slice or bytes 0: the scores do not serve (k too large, too many candidates, or FFMA is quicker)
 size_t knn_exact_left_bytes(long long nq);
 size_t knn_exact_scratch_bytes(long long n, long long nq, int d, int k, int sms);
 long long knn_exact_slice(long long n, long long nq, int d, int k, int sms);

@@ -60,7 +60,9 @@ constexpr int kAccCols = 2 * kTcN;                 // two accumulators: all 512 
 constexpr long long kWaitLimitNs = 2000000000ll;  // 2 s: no wait of a healthy launch comes near it
 constexpr long long kMaxPolls = 1ll << 26;
 constexpr int kMaxK = 96;          // k peos_knn_tensor serves (candidates per segment: k + 16)
-constexpr int kMaxCandTotal = 4096;  // candidates per query over all segments (finalize's shared memory)
+// candidates per query over all segments (finalize's shared memory); the precise form takes up
+// to four times as many where more CTAs are worth it (see tc_plan)
+constexpr int kMaxCandTotal = 4096;
 // Columns screened together, and scores a row buffers before they enter its heap (at least a
 // group): 16 and 20 per warp where 8 epilogue warps' buffers fit in shared memory beside the
 // lists, 8 and 12 with 4 warps (long lists).
@@ -906,7 +908,7 @@ int tc_pitch(int d) { return (d + kTcK - 1) / kTcK * kTcK; }
 
 // The plan of one call: how the tiles are shared and what the scratch holds.
 struct TcPlan {
-  int pitch, cand, nseg, slabs;
+  int pitch, cand, nseg, slabs, most_cand;
   long long slab_rows;  // base rows converted at a time
   TcShare share;        // of a full slab
   size_t xb, qb, xnorm, cand_buf, flags, total;  // scratch offsets
@@ -935,7 +937,7 @@ int tc_slices(long long n, long long qt, int cand, int sms) {
   return (int)best;
 }
 
-TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, int sms) {
+TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, int most_cand, int sms) {
   TcShare s;
   const long long qt = (nq + kTcM - 1) / kTcM;
   s.bt = (int)((n + kTcN - 1) / kTcN);
@@ -948,11 +950,11 @@ TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, i
     s.st = (int)(((n + want - 1) / want + kTcN - 1) / kTcN);
     s.ns = (s.bt + s.st - 1) / s.st;
   }
-  // one CTA per SM; no more than kMaxCandTotal candidates per query over its segments (a
+  // one CTA per SM; no more than most_cand candidates per query over its segments (a
   // query tile's share spans at most ceil(G / qt) + 1 CTAs), and segments of at least 4
   // tiles, below which the lists' start-up would outweigh the tiles
   long long G = sms;
-  const long long most = kMaxCandTotal / ((long long)cand * slabs);
+  const long long most = most_cand / ((long long)cand * slabs);
   const long long room = most - s.ns + 1;  // lists of a query tile beside its slices' own
   if (room >= 2) G = std::min(G, std::max(1LL, (room - 1) * qt));
   else G = std::min(G, qt);
@@ -979,6 +981,34 @@ constexpr int kMaxCand = 113;
 // the base is converted in slabs of at most 768 MiB, the rest holds queries and lists.
 constexpr size_t kExactBytes = (size_t)1 << 30, kExactSlabBytes = (size_t)768 << 20;
 
+// Estimated times of the exact brute force in us, from the measured rates of both forms: per
+// tile of 256 rows and 128 queries 0.9 + 2.1 us for every 128 elements of a row (a fifth more
+// where the query tile does not stay in shared memory, 1.4 times with 4 epilogue warps), 0.7 us
+// per insertion into a list, finalize's sort in steps of 512 keys, and the conversion at
+// 5.5 TB/s; a FFMA chunk of 16,384 rows by its 10.4 us per element, by its insertions, and 1.25
+// of them at once on an SM.  Against 94 measured shapes (2,048..10M rows, d = 4..960, 1..10,000
+// queries, k = 1..105) the FFMA estimates are 0.68..1.30 of the time and the scores' 0.36..1.72
+// (lowest for 10,000 queries over few rows, where the other form is far off), and the quicker
+// form is chosen in all but one (2,048 x 4, one query, k = 10: 112 us against 94).
+double exact_us(const TcPlan& p, long long n, long long nq, int d, int k, int sms) {
+  const double qt = (double)((nq + kTcM - 1) / kTcM), G = p.share.G;
+  const double wide = p.cand > 84 ? 1.4 : 1.0;  // 4 epilogue warps beside lists that long
+  const double tile = (0.9 + 2.1 * p.pitch / 128 * (p.pitch > 256 ? 1.2 : 1.0)) * wide;
+  const double rows = std::min((double)p.slab_rows, std::max(256.0, p.slab_rows * qt / G));
+  const double ins = p.cand * (1.0 + log(std::max(1.0, rows / p.cand)));
+  int lg = 1;
+  while ((1 << lg) < p.nseg * p.cand) ++lg;
+  const double sort = 0.5 * lg * (lg + 1) * (1 << lg) / 512 * std::max(1.0, (double)nq / sms);
+  const double finalize = lg <= 10 && nq >= 2LL * sms ? 0.025 * sort : 0.05 * sort;
+  return 65.0 + n * (4.0 * d + 4.0 * p.pitch) / 5.5e6 +
+         p.slabs * (p.share.units / G * tile + (G + qt - 1.0) / G * 0.7 * ins) + finalize;
+}
+double ffma_us(long long n, long long nq, int d, int k, int sms) {
+  const double rows = (double)std::min(n, 16384LL), ctas = (double)((n + 16383) / 16384) * ((nq + 31) / 32);
+  const double chunk = rows / 16384 * (10.4 * d + 90.0) + k * (1.0 + log(std::max(1.0, rows / k))) * (0.6 + 0.008 * k);
+  return 45.0 + chunk * std::max(1.0, ctas / sms / 1.25);
+}
+
 // False: not served.
 bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcPlan* p) {
   p->pitch = tc_pitch(d);
@@ -992,14 +1022,23 @@ bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcP
     p->slabs = (int)((n + fit - 1) / fit);
     p->slab_rows = p->slabs > 1 ? fit : n;
   }
-  p->share = tc_share(p->slab_rows, nq, p->cand, p->slabs, precise, sms);
-  int seg = p->share.max_segments();
-  if (p->slabs > 1) {
-    const TcShare last = tc_share(n - (long long)(p->slabs - 1) * p->slab_rows, nq, p->cand, p->slabs, precise, sms);
-    seg = std::max(seg, last.max_segments());
+  bool served = false;
+  TcPlan best = *p;
+  for (int most = kMaxCandTotal; most <= (precise ? 4 : 1) * kMaxCandTotal; most *= 2) {
+    p->most_cand = most;
+    p->share = tc_share(p->slab_rows, nq, p->cand, p->slabs, precise, most, sms);
+    int seg = p->share.max_segments();
+    if (p->slabs > 1) {
+      const TcShare last = tc_share(n - (long long)(p->slabs - 1) * p->slab_rows, nq, p->cand, p->slabs, precise, most, sms);
+      seg = std::max(seg, last.max_segments());
+    }
+    p->nseg = seg * p->slabs;
+    if ((long long)p->nseg * p->cand > most && p->nseg > 1) continue;
+    if (!served || exact_us(*p, n, nq, d, k, sms) < exact_us(best, n, nq, d, k, sms)) best = *p;
+    served = true;
   }
-  p->nseg = seg * p->slabs;
-  if ((long long)p->nseg * p->cand > kMaxCandTotal && p->nseg > 1) return false;
+  if (!served) return false;
+  *p = best;
   size_t o = 0;
   p->xb = o;
   o += up256((size_t)p->slab_rows * row);
@@ -1077,7 +1116,7 @@ cudaError_t run_tc(const TcPlan& p, const float* X, long long n, int d, const fl
     ta.xnorm = xnorm;
     ta.n = rows;
     ta.nq = nq;
-    ta.share = rows == p.slab_rows ? p.share : tc_share(rows, nq, p.cand, p.slabs, PRECISE, sms);
+    ta.share = rows == p.slab_rows ? p.share : tc_share(rows, nq, p.cand, p.slabs, PRECISE, p.most_cand, sms);
     ta.kchunks = p.pitch / kTcK;
     ta.cand = p.cand;
     ta.row0 = (uint32_t)r0;
@@ -1162,9 +1201,14 @@ namespace {
 size_t left_bytes(long long nq) { return kTcPad + up256((size_t)nq * 4); }
 }  // namespace
 
+// Where the FFMA form is quicker the scores do not serve: a few queries over a large base (their
+// lists limit the CTAs: 10M x 128, k = 100, 1 / 32 queries 13.1 / 18.2 ms against 8.5 / 8.6;
+// 10M x 960, k = 10, one query 76 against 41), and short rows of a small one (2,048 x 4, k = 10,
+// 1 / 500 / 10,000 queries 94 / 161 / 284 us against 112 / 130 / 170).
 size_t knn_exact_scratch_bytes(long long n, long long nq, int d, int k, int sms) {
   TcPlan p;
-  return tc_plan(n, nq, d, k, true, sms, &p) ? left_bytes(nq) + p.total : 0;
+  if (!tc_plan(n, nq, d, k, true, sms, &p) || exact_us(p, n, nq, d, k, sms) >= ffma_us(n, nq, d, k, sms)) return 0;
+  return left_bytes(nq) + p.total;
 }
 
 long long knn_exact_slice(long long n, long long nq, int d, int k, int sms) {
