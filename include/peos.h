@@ -498,6 +498,12 @@ peos_status peos_selftest_bounded_wait(int64_t limit_us, int32_t* gave_up, void*
 peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* queries, int32_t k,
                                 int32_t* ids_out, float* dists_out, void* stream);
 
+/* Self-test of the exact brute force: peos_knn_bruteforce on these arguments, and how many of
+ * its queries the tensor-core scores could not prove and left to the FFMA kernel (*left, host;
+ * -1 where the scores do not serve and it takes all of them).  Synchronises `stream`. */
+peos_status peos_selftest_knn_left(const peos_matrix* base, const peos_matrix* queries, int32_t k, int32_t* ids_out,
+                                   float* dists_out, int64_t* left, void* stream);
+
 /* Device-time tracing of the search stages (diagnostics and the benchmark's roofline).
  * Stages: set-up (the descending-efs order of an uneven batch), the search kernel, the
  * FP32 re-rank.  While tracing is on, every search call records CUDA events on its

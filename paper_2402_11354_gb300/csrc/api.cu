@@ -1073,8 +1073,9 @@ peos_status peos_selftest_bounded_wait(int64_t limit_us, int32_t* gave_up, void*
 // 300,000 rows 1.5 / 6.8 ms against 0.23 / 0.89; below, the six launches cost what one does).
 static constexpr int64_t kKnnExactMinRows = 2048;
 
-peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* queries, int32_t k, int32_t* ids_out,
-                                float* dists_out, void* stream) {
+// left (or null): the queries left to the FFMA kernel, -1 where it takes all of them; waits for them
+static peos_status knn_exact(const peos_matrix* base, const peos_matrix* queries, int32_t k, int32_t* ids_out,
+                             float* dists_out, void* stream, int64_t* left) {
   NvtxRange nvtx_range("peos.knn");
   peos_status st = check_matrix(base, "base");
   if (st) return st;
@@ -1084,6 +1085,7 @@ peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* quer
   if (k < 1 || k > 256) return set_error(PEOS_E_INVAL, "k must be in 1..256");
   if (base->n < 1) return set_error(PEOS_E_INVAL, "empty base");
   if (queries->n > 0 && (!ids_out || !dists_out)) return set_error(PEOS_E_INVAL, "NULL output");
+  if (left) *left = -1;
   if (queries->n == 0) return PEOS_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // the FFMA form's per-chunk lists take nq x chunks x k keys: its queries go in slices whose
@@ -1125,6 +1127,13 @@ peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* quer
     e = cudaErrorNotSupported;
     if (exact && knn_exact_scratch_bytes(base->n, nq, base->d, k, sms))
       e = launch_knn_exact(X, base->n, base->d, q, nq, k, ids, dists, scratch.p, slice, sms, s);
+    if (left && e == cudaSuccess) {
+      int32_t count = 0;
+      e = cudaMemcpyAsync(&count, static_cast<const int32_t*>(scratch.p) + 1, sizeof(count), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) return cuda_error(e, "knn left-over count");
+      *left = std::max<int64_t>(*left, 0) + count;
+    }
     if (e == cudaErrorNotSupported) {  // also where tensor maps are not available
       e = cudaSuccess;
       for (int64_t o = 0; o < nq && e == cudaSuccess; o += slice)
@@ -1134,6 +1143,17 @@ peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* quer
     if (e != cudaSuccess) return cuda_error(e, "knn launch");
   }
   return PEOS_OK;
+}
+
+peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* queries, int32_t k, int32_t* ids_out,
+                                float* dists_out, void* stream) {
+  return knn_exact(base, queries, k, ids_out, dists_out, stream, nullptr);
+}
+
+peos_status peos_selftest_knn_left(const peos_matrix* base, const peos_matrix* queries, int32_t k, int32_t* ids_out,
+                                   float* dists_out, int64_t* left, void* stream) {
+  if (!left) return set_error(PEOS_E_INVAL, "left is NULL");
+  return knn_exact(base, queries, k, ids_out, dists_out, stream, left);
 }
 
 }  // extern "C"

@@ -2,8 +2,9 @@
 // for large bases, in two precisions of the scores.
 //
 //   1. convert: base and queries to BF16 rows (zero-padded to a multiple of 64 elements),
-//      and ||x||^2 of every base row in FP32.  The precise form keeps each value as the sum
-//      of two BF16 terms, hi and lo, in a row of twice the length.
+//      and ||x||^2 of every base row in FP32.  The precise form takes a centre of the base
+//      off every row and keeps each value as the sum of two BF16 terms, hi and lo, in a row
+//      of twice the length.
 //   2. candidates: one CTA per SM takes an equal, contiguous share of the (128 queries x 256
 //      base rows) tiles, query tile by query tile; a query tile that spans CTAs has one
 //      candidate list per CTA (a segment).  A TMA warp brings 128 x 64 query and 256 x 64 base
@@ -174,68 +175,118 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// The precise form works on rows less a centre of the base, so that the score's error is
+// relative to the rows' spread and not to a common offset.  Per coordinate the mean of five
+// medians of three rows each, which one long row does not move; zero where that is no moderate
+// number.  Four coordinates from k on.  Every CTA of the queries' conversion finds it for itself
+// (16,384 x 100, one query: 112 us for the call; a launch of its own 117).
+__device__ __forceinline__ float median3(float a, float b, float c) { return fmaxf(fminf(a, b), fminf(fmaxf(a, b), c)); }
+__device__ __forceinline__ float4 centre_of(const float* __restrict__ X, long long n, int d, int k) {
+  float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int j = 0; j < 15; j += 3) {
+    float4 v[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v[i] = __ldg(reinterpret_cast<const float4*>(X + (size_t)(n * (j + i) / 15) * d + k));
+    m.x += median3(v[0].x, v[1].x, v[2].x);
+    m.y += median3(v[0].y, v[1].y, v[2].y);
+    m.z += median3(v[0].z, v[1].z, v[2].z);
+    m.w += median3(v[0].w, v[1].w, v[2].w);
+  }
+  auto moderate = [](float x) { return fabsf(x) < 1e18f ? 0.2f * x : 0.0f; };
+  return make_float4(moderate(m.x), moderate(m.y), moderate(m.z), moderate(m.w));
+}
+
 // A warp takes four rows at a time (their loads in flight together), four elements per lane.
-// LO: the rounding errors' own BF16 values follow the row's hi terms.  norm2: FP32 squared
+// LO: rows less `centre` (FIND, the queries: found here, and stored; the call's flags are
+// cleared); the rounding errors' own BF16 values follow the row's hi terms.  norm2: FP32 squared
 // norms (base rows); xmax: the largest of them, as its bits (a NaN's bits are larger than any
 // number's).  Without LO: `inexact` is set when a score of these rows may be rounded: an
 // element that is not an integer of at most 256, or a squared norm of 2^24 / 3 or more (below,
 // ||x||^2 + 2 |q.x| and all sums on the way stay under 2^24).
 constexpr float kExactNorm2 = 5.5e6f;
-template <bool LO>
+constexpr int kConvertThreads = 256;
+template <bool LO, bool FIND>
 __global__ void convert_bf16_kernel(const float* __restrict__ X, long long n, int d, int pitch,
                                     __nv_bfloat16* __restrict__ out, float* __restrict__ norm2,
-                                    unsigned* __restrict__ xmax, unsigned* __restrict__ inexact) {
+                                    unsigned* __restrict__ xmax, unsigned* __restrict__ inexact,
+                                    float* __restrict__ centre, const float* __restrict__ base, long long nbase,
+                                    int* __restrict__ err) {
   constexpr int kAtOnce = 4;
+  constexpr int kWindow = 4 * kConvertThreads;  // FIND (no norms): coordinates whose centre is held at a time
+  __shared__ float4 s_centre[FIND ? kConvertThreads : 1];
   const int lane = threadIdx.x & 31;
   const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   const size_t row = (size_t)pitch * (LO ? 2 : 1);
   unsigned most = 0;
   bool rounded = false;
-  for (long long r0 = w0 * kAtOnce; r0 < n; r0 += nw * kAtOnce) {
-    float s[kAtOnce];
+  if (FIND && blockIdx.x == 0 && threadIdx.x == 0) {
+    xmax[0] = inexact[0] = 0u;
+    err[0] = err[1] = 0;
+  }
+  for (int first = 0; first < pitch; first += kWindow) {
+    const int end = FIND ? min(pitch, first + kWindow) : pitch;
+    if (FIND) {
+      __syncthreads();
+      const int k = first + 4 * threadIdx.x;
+      if (k < end) {
+        const float4 c = k < d ? centre_of(base, nbase, d, k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        s_centre[threadIdx.x] = c;
+        if (blockIdx.x == 0) *reinterpret_cast<float4*>(centre + k) = c;
+      }
+      __syncthreads();
+    }
+    for (long long r0 = w0 * kAtOnce; r0 < n; r0 += nw * kAtOnce) {
+      float s[kAtOnce];
 #pragma unroll
-    for (int j = 0; j < kAtOnce; ++j) s[j] = 0.0f;
-    for (int k = 4 * lane; k < pitch; k += 128) {
-      float4 v[kAtOnce];
+      for (int j = 0; j < kAtOnce; ++j) s[j] = 0.0f;
+      for (int k = first + 4 * lane; k < end; k += 128) {
+        float4 v[kAtOnce];
 #pragma unroll
-      for (int j = 0; j < kAtOnce; ++j)
-        v[j] = (k < d && r0 + j < n) ? __ldg(reinterpret_cast<const float4*>(X + (size_t)(r0 + j) * d + k))
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int j = 0; j < kAtOnce; ++j)
+          v[j] = (k < d && r0 + j < n) ? __ldg(reinterpret_cast<const float4*>(X + (size_t)(r0 + j) * d + k))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 ce = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (FIND) ce = s_centre[(k - first) >> 2];
+        else if (LO) ce = __ldg(reinterpret_cast<const float4*>(centre + k));
 #pragma unroll
-      for (int j = 0; j < kAtOnce; ++j) {
-        if (r0 + j >= n) break;
-        const float4 x = v[j];
-        const uint2 h = make_uint2(bf16_pair(x.x, x.y), bf16_pair(x.z, x.w));
-        __nv_bfloat16* o = out + (size_t)(r0 + j) * row + k;
-        *reinterpret_cast<uint2*>(o) = h;
-        if (LO) {
-          const float4 f = make_float4(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xffff0000u),
-                                       __uint_as_float(h.y << 16), __uint_as_float(h.y & 0xffff0000u));
-          *reinterpret_cast<uint2*>(o + pitch) =
-              make_uint2(bf16_pair(x.x - f.x, x.y - f.y), bf16_pair(x.z - f.z, x.w - f.w));
+        for (int j = 0; j < kAtOnce; ++j) {
+          if (r0 + j >= n) break;
+          float4 x = v[j];
+          if (LO) x = make_float4(x.x - ce.x, x.y - ce.y, x.z - ce.z, x.w - ce.w);
+          const uint2 h = make_uint2(bf16_pair(x.x, x.y), bf16_pair(x.z, x.w));
+          __nv_bfloat16* o = out + (size_t)(r0 + j) * row + k;
+          *reinterpret_cast<uint2*>(o) = h;
+          if (LO) {
+            const float4 f = make_float4(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xffff0000u),
+                                         __uint_as_float(h.y << 16), __uint_as_float(h.y & 0xffff0000u));
+            *reinterpret_cast<uint2*>(o + pitch) =
+                make_uint2(bf16_pair(x.x - f.x, x.y - f.y), bf16_pair(x.z - f.z, x.w - f.w));
+          }
+          s[j] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+          if (!LO) {
+            const float top = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w)));
+            // adding 1.5 2^23 rounds to an integer (of small values; larger ones fail the other test)
+            const float e = fabsf(((x.x + 12582912.0f) - 12582912.0f) - x.x) + fabsf(((x.y + 12582912.0f) - 12582912.0f) - x.y) +
+                            fabsf(((x.z + 12582912.0f) - 12582912.0f) - x.z) + fabsf(((x.w + 12582912.0f) - 12582912.0f) - x.w);
+            rounded = rounded || !(e == 0.0f && top <= 256.0f);
+          }
         }
-        s[j] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
-        if (!LO) {
-          const float top = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w)));
-          // adding 1.5 2^23 rounds to an integer (of small values; larger ones fail the other test)
-          const float e = fabsf(((x.x + 12582912.0f) - 12582912.0f) - x.x) + fabsf(((x.y + 12582912.0f) - 12582912.0f) - x.y) +
-                          fabsf(((x.z + 12582912.0f) - 12582912.0f) - x.z) + fabsf(((x.w + 12582912.0f) - 12582912.0f) - x.w);
-          rounded = rounded || !(e == 0.0f && top <= 256.0f);
+      }
+      if (norm2 || !LO) {
+#pragma unroll
+        for (int j = 0; j < kAtOnce; ++j) {
+          const float t = warp_sum(s[j]);
+          rounded = rounded || !(t < kExactNorm2);
+          if (norm2 && r0 + j < n) {
+            if (lane == 0) norm2[r0 + j] = t;
+            most = max(most, __float_as_uint(t));
+          }
         }
       }
     }
-    if (norm2 || !LO) {
-#pragma unroll
-      for (int j = 0; j < kAtOnce; ++j) {
-        const float t = warp_sum(s[j]);
-        rounded = rounded || !(t < kExactNorm2);
-        if (norm2 && r0 + j < n) {
-          if (lane == 0) norm2[r0 + j] = t;
-          most = max(most, __float_as_uint(t));
-        }
-      }
-    }
+    if (!FIND) break;
   }
   if (!LO && __any_sync(kFull, rounded) && lane == 0) *inexact = 1u;
   if (norm2 && lane == 0 && most) atomicMax(xmax, most);
@@ -718,8 +769,10 @@ struct FinArgs {
   int32_t* ids_out;
   float* dists_out;
   const unsigned* xmax;  // bits of the largest ||x||^2
-  float c_dot;           // |score error| <= c_dot ||q|| ||x||max + c_norm ||x||max^2
-  float c_norm;
+  const float* centre;   // precise form: what was taken off rows and queries
+  float c_dot;           // |score error| <= c_dot ||q|| ||x|| + c_norm ||x||^2 + c_q ||q||^2
+  float c_norm, c_q;
+  float reach;           // see `radius` below
   // precise form: queries whose result is not proven
   const int* err;
   int* left_count;
@@ -764,18 +817,30 @@ __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_fina
   const int t = WPQ == 1 ? lane : threadIdx.x;
   uint64_t* s_key = reinterpret_cast<uint64_t*>(smem_raw) + (size_t)(WPQ == 1 ? warp : 0) * a.P;
   const int d = a.d, d4 = d >> 2, ncand = a.nseg * a.ncand1;
-  const double xm2 = (double)__uint_as_float(*a.xmax), xm = sqrt(xm2);
+  const float xm2 = __uint_as_float(*a.xmax), xm = 1.00001f * sqrtf(xm2);
   for (long long q = (long long)blockIdx.x * kQueries + (WPQ == 1 ? warp : 0); q < a.nq; q += (long long)gridDim.x * kQueries) {
     const float4* qv = reinterpret_cast<const float4*>(a.Q + (size_t)q * d);
-    // ||q||^2, the same in every warp
+    // ||q||^2 (less the centre), the same in every warp
     double q2 = 0.0;
     for (int c = lane; c < d4; c += 32) {
-      const float4 v = __ldg(qv + c);
+      float4 v = __ldg(qv + c);
+      if (PRECISE) {
+        const float4 ce = __ldg(reinterpret_cast<const float4*>(a.centre) + c);
+        v = make_float4(v.x - ce.x, v.y - ce.y, v.z - ce.z, v.w - ce.w);
+      }
       q2 += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q2 += __shfl_xor_sync(kFull, q2, o);
-    const double err = (double)a.c_dot * sqrt(q2) * xm + (double)a.c_norm * xm2;
+    const float qn = 1.00001f * sqrtf((float)q2);
+    // The score's error for a row of norm up to r.  Only rows near the query matter: one of norm
+    // N > 2 (||q|| + sqrt(D)) lies N / 2 + sqrt(D) or more from the query, beyond a distance of D
+    // whatever its score's error, and scores above D - ||q||^2 as long as that error is below
+    // N^2 / 4 (reach: 2, or infinity where it may not be).  So one long row does not widen the bound.
+    // Both in FP32, rounded up, with room for values that underflow (in FP64, which is slow here,
+    // 6.27 ms against 6.10: 65,536 x 960, 10,000 queries, k = 100).
+    auto error_to = [&](float r) { return 1.0001f * (a.c_dot * qn * r + a.c_norm * r * r + a.c_q * qn * qn) + 1e-30f; };
+    auto radius = [&](double D) { return fminf(xm, a.reach * (qn + 1.0001f * sqrtf(fmaxf((float)D, 0.0f))) + 1e-12f); };
     const uint64_t* src = a.cand + (size_t)q * ncand;
     int P = a.P;
     if (WPQ == 1 && !PRECISE) {  // the filled slots alone
@@ -805,7 +870,11 @@ __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_fina
     // also in FP32
     const double fp = (double)(d + 4) * 0x1p-23;
     const uint64_t kth = s_key[a.k - 1];
-    const double thr = kth == kNoKey ? INFINITY : (double)key_score(kth) + 2.0 * err + fp * fabs((double)key_score(kth) + err + q2);
+    double thr = INFINITY;
+    if (kth != kNoKey) {
+      const double S = (double)key_score(kth), err = (double)error_to(radius(S + q2)), D = S + err + q2;
+      thr = S + err + (double)error_to(radius(D)) + fp * fabs(D);
+    }
     int m = 0;  // candidates to measure: the first m
     {
       int lo = 0, hi = P;
@@ -866,11 +935,12 @@ __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_fina
     if (PRECISE && t == 0) {
       // below 1e37 no score, no BF16 term and no distance overflows (|q.x| <= ||q|| ||x||); a
       // score that did would have entered no list
-      bool proven = *a.err == 0 && xm2 >= 1e-24 && xm2 < 1e37 && (q2 >= 1e-24 || q2 == 0.0) && q2 < 1e37;
+      bool proven = *a.err == 0 && xm2 >= 1e-24f && xm2 < 1e37f && (q2 >= 1e-24 || q2 == 0.0) && q2 < 1e37;
       if (left_out != kNoKey) {
         const uint64_t last = s_key[a.k - 1];
         proven = proven && last != kNoKey &&
-                 ((double)key_score(left_out) - err + q2) * (1.0 - fp) > (double)key_dist(last) * (1.0 + 0x1p-20);
+                 ((double)key_score(left_out) - (double)error_to(radius((double)key_dist(last))) + q2) * (1.0 - fp) >
+                     (double)key_dist(last) * (1.0 + 0x1p-20);
       }
       if (!proven) a.left[atomicAdd(a.left_count, 1)] = (int32_t)q;
     }
@@ -921,7 +991,7 @@ struct TcPlan {
   int pitch, cand, nseg, slabs, most_cand;
   long long slab_rows;  // base rows converted at a time
   TcShare share;        // of a full slab
-  size_t xb, qb, xnorm, cand_buf, flags, total;  // scratch offsets
+  size_t xb, qb, xnorm, cand_buf, centre, flags, total;  // scratch offsets
 };
 
 // cost of a list's start in tiles: it takes about cand (1 + ln(rows / cand)) insertions
@@ -1058,6 +1128,8 @@ bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcP
   o += up256((size_t)p->slab_rows * 4);
   p->cand_buf = o;
   o += up256((size_t)nq * p->nseg * p->cand * 8);
+  p->centre = o;
+  if (precise) o += up256((size_t)p->pitch * 4);
   p->flags = o;  // xmax, inexact
   o += kTcPad;
   p->total = o;
@@ -1105,19 +1177,20 @@ cudaError_t run_tc(const TcPlan& p, const float* X, long long n, int d, const fl
   float* xnorm = reinterpret_cast<float*>(w + p.xnorm);
   uint64_t* cand_buf = reinterpret_cast<uint64_t*>(w + p.cand_buf);
   unsigned* xmax = reinterpret_cast<unsigned*>(w + p.flags);
+  float* centre = PRECISE ? reinterpret_cast<float*>(w + p.centre) : nullptr;
   cudaError_t e = cudaMemsetAsync(cand_buf, 0xff, (size_t)nq * p.nseg * p.cand * 8, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(xmax, 0, 2 * sizeof(unsigned), st);
+  if (!PRECISE && e == cudaSuccess) e = cudaMemsetAsync(xmax, 0, 2 * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   const int cols = p.pitch * (PRECISE ? 2 : 1);
   const int cg = sms * 8;
-  convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (nq + 31) / 32), 256, 0, st>>>(Q, nq, d, p.pitch, qb,
-                                                                                               nullptr, nullptr, xmax + 1);
+  convert_bf16_kernel<PRECISE, PRECISE><<<(unsigned)std::min<long long>(cg, (nq + 31) / 32), kConvertThreads, 0, st>>>(
+      Q, nq, d, p.pitch, qb, nullptr, xmax, xmax + 1, centre, X, n, err);
   CUtensorMap mq;
   if (!make_map(&mq, qb, nq, cols, kTcM)) return cudaErrorNotSupported;
   for (int s = 0; s < p.slabs; ++s) {
     const long long r0 = (long long)s * p.slab_rows, rows = std::min(p.slab_rows, n - r0);
-    convert_bf16_kernel<PRECISE><<<(unsigned)std::min<long long>(cg, (rows + 31) / 32), 256, 0, st>>>(
-        X + (size_t)r0 * d, rows, d, p.pitch, xb, xnorm, xmax, xmax + 1);
+    convert_bf16_kernel<PRECISE, false><<<(unsigned)std::min<long long>(cg, (rows + 31) / 32), kConvertThreads, 0, st>>>(
+        X + (size_t)r0 * d, rows, d, p.pitch, xb, xnorm, xmax, xmax + 1, centre, nullptr, 0, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     CUtensorMap mx;
@@ -1156,13 +1229,22 @@ cudaError_t run_tc(const TcPlan& p, const float* X, long long n, int d, const fl
   fa.ids_out = ids_out;
   fa.dists_out = dists_out;
   fa.xmax = xmax;
+  fa.centre = centre;
   // Score error, relative to ||q|| ||x||: the terms dropped or rounded (BF16's unit roundoff
   // is 2^-8: 2 (2^-8 + 2^-18) alone, 3.05 2^-16 for the two-term sums), and the FP32
   // accumulation, at most 2^-23 per product (each step of 16 aligns its products and the
   // accumulator to the largest and truncates); times 2 for -2 q.x, plus the last rounding.
+  // Taking the centre off rounds every element once: x and q move by at most 2^-24 of their
+  // norms, their squared distance by 2^-23 (||x|| + ||q||)^2.
   const double products = (double)p.pitch * (PRECISE ? 3 : 1);
   fa.c_dot = (float)(2.0 * ((PRECISE ? 3.05 * 0x1p-16 : 2.02 * 0x1p-8) + products * 0x1p-23) + 0x1p-21);
   fa.c_norm = (float)((d / 32 + 10) * 0x1p-23);
+  if (PRECISE) {
+    fa.c_dot += 1.01f * 0x1p-22f;
+    fa.c_norm += 1.01f * 0x1p-23f;
+    fa.c_q = 1.01f * 0x1p-23f;
+  }
+  fa.reach = 0.5f * fa.c_dot + fa.c_norm + fa.c_q < 0.2f ? 2.0f : INFINITY;
   fa.err = err;
   fa.left_count = left_count;
   fa.left = left;
@@ -1238,9 +1320,7 @@ cudaError_t launch_knn_exact(const float* X, long long n, int d, const float* Q,
   int* left_count = err + 1;
   int32_t* left = reinterpret_cast<int32_t*>(static_cast<unsigned char*>(scratch) + kTcPad);
   unsigned char* w = static_cast<unsigned char*>(scratch) + left_bytes(nq);
-  cudaError_t e = cudaMemsetAsync(err, 0, 2 * sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  e = run_tc<true>(p, X, n, d, Q, nq, k, ids_out, dists_out, w, err, left_count, left, sms, st);
+  cudaError_t e = run_tc<true>(p, X, n, d, Q, nq, k, ids_out, dists_out, w, err, left_count, left, sms, st);
   // the scores are done with w when these run; all but the list's own are empty launches
   for (long long q = 0; q < nq && e == cudaSuccess; q += ffma_slice)
     e = launch_knn(X, n, d, Q, std::min(ffma_slice, nq - q), k, ids_out, dists_out, w, st, left, left_count, q);

@@ -86,7 +86,7 @@ def load(build_if_missing: bool = True):
                  "peos_server_stats", "peos_server_destroy", "peos_knn_tensor",
                  "peos_release_workspace", "peos_edge_stats", "peos_projections", "peos_knn_bruteforce",
                  "peos_dim_permutation", "peos_build_codes_permuted", "peos_hier_entry", "peos_build_simhash", "peos_search_host_async",
-                 "peos_selftest_bounded_wait", "peos_crc32", "peos_codes_save", "peos_codes_load", "peos_codes_graph", "peos_check_read",
+                 "peos_selftest_bounded_wait", "peos_selftest_knn_left", "peos_crc32", "peos_codes_save", "peos_codes_load", "peos_codes_graph", "peos_check_read",
                  "peos_build_codes_compact"):
         getattr(lib, name).restype = ctypes.c_int
     _lib = lib
@@ -678,6 +678,23 @@ def selftest_bounded_wait(limit_us: int = 1000, stream=None) -> bool:
     gave_up = ctypes.c_int32(-1)
     _check(load().peos_selftest_bounded_wait(ctypes.c_int64(limit_us), ctypes.byref(gave_up), _stream(stream)))
     return gave_up.value == 1
+
+
+def selftest_knn_left(base: torch.Tensor, queries: torch.Tensor, k: int, stream=None) -> int:
+    """How many queries of knn_bruteforce(base, queries, k) the tensor-core scores could not
+    prove and left to the FFMA kernel; -1 where that kernel takes all of them."""
+    base = _dev_f32(base, "base")
+    queries = _dev_f32(queries, "queries")
+    nq = queries.shape[0]
+    ids = torch.empty((nq, k), dtype=torch.int32, device=queries.device)
+    dists = torch.empty((nq, k), dtype=torch.float32, device=queries.device)
+    Mb, Mq = _matrix(base), _matrix(queries)
+    left = ctypes.c_int64(-1)
+    _check(load().peos_selftest_knn_left(ctypes.byref(Mb), ctypes.byref(Mq), ctypes.c_int32(k),
+                                         ctypes.c_void_p(ids.data_ptr() if nq else 0),
+                                         ctypes.c_void_p(dists.data_ptr() if nq else 0), ctypes.byref(left),
+                                         _stream(stream)))
+    return left.value
 
 
 CHECK_KINDS = ["candidate", "expanded", "list_write", "list_order", "list_duplicate"]
