@@ -805,14 +805,15 @@ __device__ __forceinline__ void group_sort(uint64_t* key, int P, int t) {
 }
 
 constexpr int kFinWarps = 4;      // warps per CTA where a warp takes a query
-// 16-byte pieces of a candidate's row loaded at a time (65,536 x 960, 10,000 queries, k = 100:
-// 1.32 ms; 8 pieces 1.42, and 1.3 to 2.3 where the compiler chooses)
-constexpr int kAhead = 4;
 constexpr int kFinGroupWarps = 8;  // where a CTA takes one
 template <int WPQ, bool PRECISE>
 __global__ void __launch_bounds__((WPQ == 1 ? kFinWarps : WPQ) * 32) knn_tc_finalize(FinArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int kQueries = WPQ == 1 ? kFinWarps : 1;  // per CTA
+  // 16-byte pieces of a candidate's row loaded at a time, 4 / 8: a warp per query 1.32 / 1.42 ms
+  // (65,536 x 960, 10,000 queries, k = 100; 1.3 to 2.3 where the compiler chooses), a CTA per query
+  // 0.239 / 0.219 (300,000 x 100, 2,000 queries, k = 100)
+  constexpr int kAhead = WPQ == 1 ? 4 : 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = WPQ == 1 ? lane : threadIdx.x;
   uint64_t* s_key = reinterpret_cast<uint64_t*>(smem_raw) + (size_t)(WPQ == 1 ? warp : 0) * a.P;
