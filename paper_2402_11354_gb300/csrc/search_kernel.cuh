@@ -813,13 +813,15 @@ __global__ void __launch_bounds__(kMaxWarps * 32, Shape<G>::kMinCtas) search_ker
         //      candidate before it did and dist < the (ef-1-g)-th entry of R (entries past
         //      len count as +inf); J = number entering
         const bool keep0 = (km[0] >> lane) & 1u;
-        bool enters = false;
+        int fail_rank = 0x7fffffff;
         if (keep0) {
           const int idx = ef - 1 - rank;
           const float bound = idx < 0 ? -INFINITY : (idx < len ? s_rd[idx] : INFINITY);
-          enters = key_dist(key[0]) < bound;
+          if (!(key_dist(key[0]) < bound)) fail_rank = rank;
         }
-        J = __popc(__ballot_sync(kFull, enters));  // the first J by rank: the bound falls as the rank grows
+        // by rank and not by count: a list that ends in NaN (the entry's) has no falling bounds
+        J = min(nkeep, __reduce_min_sync(kFull, fail_rank));
+        const bool enters = keep0 && rank < J;
         if (J == 0) continue;
         if (ef <= 64) {
           // ---- merge of a short list: F = the slots the candidates take (position + rank); a
