@@ -482,10 +482,12 @@ peos_status peos_hier_entry(const peos_hierarchy* hierarchy, const peos_matrix* 
 
 /* Self-test of the failure detection of the library's waits: every spin-wait in the
  * device code (the tensor-core brute force's mbarrier waits) gives up after a bounded
- * time (2 s of the GPU's global timer), records the failure and returns (the host then
- * reports PEOS_E_TIMEOUT) instead of hanging.  This runs one such wait, limited to
- * `limit_us` microseconds (1..2,000,000), on an mbarrier that nothing arrives on,
- * synchronises `stream`, and sets *gave_up (host) to 1 when the wait gave up as it must.
+ * time (2 s of the GPU's global timer), records the failure and returns instead of hanging
+ * (peos_knn_tensor then reports PEOS_E_TIMEOUT; peos_knn_bruteforce hands the queries of such a
+ * launch to its FFMA kernel, which has no waits, so that its results stand).  This runs one
+ * such wait, limited to `limit_us` microseconds (1..2,000,000), on an mbarrier that nothing
+ * arrives on, synchronises `stream`, and sets *gave_up (host) to 1 when the wait gave up as it
+ * must.
  * Nothing faults or hangs; the context stays usable. */
 peos_status peos_selftest_bounded_wait(int64_t limit_us, int32_t* gave_up, void* stream);
 
@@ -493,7 +495,11 @@ peos_status peos_selftest_bounded_wait(int64_t limit_us, int32_t* gave_up, void*
  * for each query the k base rows with the smallest squared l2 distance, ascending
  * (dist, id).  Distances are exact FP32 sums of squared differences.
  * base/queries: device PEOS_F32; ids_out [nq][k], dists_out [nq][k] device;
- * 1 <= k <= 256.  Uses library-owned scratch of at most about 1 GiB (queries and base run in
+ * 1 <= k <= 256.  From 2,048 rows on, where it is estimated to be quicker and k <= 105, the
+ * tensor cores score the rows first and a query's result is proven from the scores' error
+ * bound; the queries it cannot prove (rows repeated more often than a list of k + 16 holds,
+ * groups of rows far apart) cost the FFMA kernel's time on top.  Results are the same either
+ * way, bit for bit.  Uses library-owned scratch of at most about 1 GiB (queries and base run in
  * slices whose converted rows and candidate lists fit in it). */
 peos_status peos_knn_bruteforce(const peos_matrix* base, const peos_matrix* queries, int32_t k,
                                 int32_t* ids_out, float* dists_out, void* stream);
@@ -517,7 +523,8 @@ peos_status peos_trace_read(double* ms, int64_t* calls);
 
 /* The same K-NN on the tensor cores (tcgen05, BF16 inputs, FP32 accumulation in tensor
  * memory) for large bases: every base row is scored by ||x||^2 - 2 q.x for every query,
- * each query keeps its k + 16 best rows per slice of the base, and those candidates get
+ * each query keeps its k + 16 best rows per slice of the base (on integer-valued data below
+ * 256 per CTA that works on the query), and those candidates get
  * their exact FP32 squared distances (sequential over the dimensions) and are ranked by
  * (dist, id).  On integer-valued data below 256 the BF16 scores are exact and the result
  * is the exact K-NN; otherwise BF16 rounding can only reorder near-ties among rows the

@@ -739,8 +739,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, 1) build_edges_kernel(TileArg
 
 // ---- the screened form: blocks of 8..64 coordinates, a multiple of 4 -----------------
 //
-// A code is an argmax over 16 sums, and only that: sums good to five digits settle all but a
-// few in a thousand.  A warp takes 32 edges and forms, on the tensor cores, every e_i . a^i_j
+// A code is an argmax over 16 sums, and only that: sums good to five digits settle nearly all
+// (left: 0.13% of the block codes and 0.5% of the e[0] of 1M x 128, 0.22% and 2.6% of 50,000 x 960).  A warp takes 32 edges and forms, on the tensor cores, every e_i . a^i_j
 // and e_i . b_j (two BF16 terms of each factor, three products, mma.sync on fragments built
 // straight from the staged rows); per block it keeps the two largest |e_i . a^i_j|, and the
 // b_j sums of e_res follow from two running sums, sum_i P_i and sum_i P_i / ||e_i||, since

@@ -35,7 +35,7 @@
 //
 // Every wait on an mbarrier is bounded: after kWaitLimitNs of the global timer (or
 // kMaxPolls polls, whichever comes first) the CTA records an error and stops issuing work
-// (the host reports PEOS_E_TIMEOUT).
+// (the host reports PEOS_E_TIMEOUT; the precise form's queries go to the FFMA kernel).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>

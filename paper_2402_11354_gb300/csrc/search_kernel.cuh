@@ -338,7 +338,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, Shape<G>::kMinCtas) search_ker
   constexpr int NL = kGroups ? 1 : NR;  // edges held per lane
   // lists of up to 64 entries: the candidates' positions by a search of fixed steps (PEOs,
   // where few lanes hold a candidate: sift-shaped 440 -> 432 us, GIST-shaped 2.85 -> 2.65 ms;
-  // plain routing 404 -> 444 us, and lists of 512 7.41 -> 7.82 ms, keep the divergent search)
+  // plain routing 404 -> 444 us, and lists of 512 7.41 -> 7.82 ms, keep the divergent search).
+  // The same kernels merge longer lists 32 slots at a time.
   constexpr bool kFixedSearch = W == 1 && NL == 1 && ROUTING != 0;
   constexpr int NRC = W * NL;     // candidate registers per lane: candidate g = r * 32 + lane
   [[maybe_unused]] constexpr int kCand = NRC * 32;  // candidates one iteration can hold (checked builds)
