@@ -300,8 +300,8 @@ struct TcShare {
   int bt, G;
   int st, ns;       // tiles per slice, slices per query tile (st >= bt, 1: not sliced)
   int whole;
-  __host__ __device__ long long start(int c) const {
-    if (!whole) return units * c / G;
+  __host__ __device__ long long start(int c, bool by_slices) const {
+    if (!by_slices) return units * c / G;
     const long long s = units / bt * ns * c / G;  // the share's first slice
     return s / ns * bt + s % ns * st;
   }
@@ -309,9 +309,9 @@ struct TcShare {
   __host__ __device__ int cta_of(long long u) const { return (int)(((u + 1) * G - 1) / units); }
   // the list of the segment of CTA c that ends with unit u, among its query tile's lists: from
   // one segment to the next the slice, the CTA or both go up
-  __host__ __device__ int list_of(long long u, int c) const {
+  __host__ __device__ int list_of(long long u, int c, long long cut, bool by_slices) const {
     const long long q0 = u / bt * bt;
-    return (int)((u - q0) / st) + (whole ? 0 : c - cta_of(q0));
+    return (int)((u - q0) / cut) + (by_slices ? 0 : c - cta_of(q0));
   }
   // most lists of one query tile
   __host__ int max_segments() const {
@@ -336,6 +336,7 @@ struct TcArgs {
   int nseg, seg0;    // segments per query in `out`, and the launch's first
   uint64_t* out;     // [nq][nseg][cand] (ordered(approx) << 32 | id), prefilled with kNoKey
   const unsigned* inexact;  // 0: no score is rounded, and a list may go on past its slice
+  int equal;         // and the shares are equal ones all the same
   int* err;
 };
 
@@ -540,8 +541,10 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
   __shared__ __align__(16) float s_xn[EW][kTcN / kHalves];  // per epilogue warp: ||x||^2 of its columns' base rows
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long u0 = a.share.start(blockIdx.x), u1 = a.share.start(blockIdx.x + 1);
   const int bt = a.share.bt;
+  const bool exact = PRECISE || __ldg(a.inexact) == 0u;
+  const bool by_slices = !PRECISE && a.share.whole && !(exact && a.equal);
+  const long long u0 = a.share.start(blockIdx.x, by_slices), u1 = a.share.start(blockIdx.x + 1, by_slices);
 
   if (tid == 0) {
     s_fail = 0;
@@ -698,7 +701,7 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
       for (int j = 0; j < kNorms; ++j) xn[j] = r + 32 * j < a.n ? __ldg(a.xnorm + r + 32 * j) : INFINITY;
     };
     if (u0 < u1) load_norms((int)(u0 % bt));
-    const long long st = PRECISE || __ldg(a.inexact) == 0u ? bt : a.share.st;
+    const long long st = exact ? bt : a.share.st;
     for (long long u = u0; u < u1;) {
       const long long qt = u / bt, qe = (qt + 1) * bt;
       const long long ue = min(min(u1, qe), qt * bt + ((u - qt * bt) / st + 1) * st);
@@ -742,7 +745,7 @@ __global__ void __launch_bounds__((EW + 2) * 32, 1) knn_tc_kernel(const __grid_c
       list.flush();
       quarter_sync<EW>(quarter);
       if (ok && qt * kTcM + row < a.nq) {
-        const int seg = a.seg0 + a.share.list_of(ue - 1, blockIdx.x);
+        const int seg = a.seg0 + a.share.list_of(ue - 1, blockIdx.x, by_slices ? a.share.st : st, by_slices);
         uint64_t* o = a.out + ((size_t)(qt * kTcM + row) * a.nseg + seg) * a.cand;
         for (int i = half; i < a.cand; i += kHalves) o[i] = list.heap[(size_t)i * kRows];
       }
@@ -992,6 +995,7 @@ struct TcPlan {
   int pitch, cand, nseg, slabs, most_cand;
   long long slab_rows;  // base rows converted at a time
   TcShare share;        // of a full slab
+  int equal;            // see equal_if_exact
   size_t xb, qb, xnorm, cand_buf, centre, flags, total;  // scratch offsets
 };
 
@@ -1053,6 +1057,38 @@ TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, i
   return s;
 }
 
+// Whole slices are for scores that are rounded.  Where none is (the kernel finds out) a list goes
+// on past its slice, and equal shares are taken after all if the CTA that has most to do then has
+// less (606,000 x 128 integer rows, 11,863 queries, k = 1: 1,580 tiles at most against 1,449,
+// 3,227 us against 3,033; 6,900 rows, 3,838 queries, k = 27 keep the slices, where a CTA
+// starts one list and not two: 406 us, 577 with equal shares).
+double busiest(const TcShare& s, bool by_slices, int cand) {
+  double most = 0.0;
+  for (int c = 0; c < s.G; ++c) {
+    const long long u1 = s.start(c + 1, by_slices);
+    double cost = 0.0;
+    for (long long u = s.start(c, by_slices); u < u1;) {
+      const long long ue = std::min(u1, (u / s.bt + 1) * s.bt);
+      cost += (double)(ue - u) + list_tiles(256.0 * (ue - u), cand);
+      u = ue;
+    }
+    most = std::max(most, cost);
+  }
+  return most;
+}
+int equal_segments(TcShare s) {
+  s.whole = 0;
+  s.ns = 1;
+  return s.max_segments();
+}
+int equal_if_exact(const TcShare& s, int cand, int most_cand) {
+  // looked at where the slices' uneven numbers cost 4% of at least 256 tiles a CTA (the sums
+  // below take some 8 us of the host)
+  const long long slices = s.units / s.bt * s.ns, least = (s.units + s.G - 1) / s.G;
+  if (least < 256 || (slices + s.G - 1) / s.G * s.st * 100 < least * 104) return 0;
+  return s.whole && equal_segments(s) * cand <= most_cand && busiest(s, false, cand) < busiest(s, true, cand);
+}
+
 // The longest list whose launch fits in shared memory (4 epilogue warps, two stages of query
 // and base chunks).  The precise form serves k up to 8 below it: its lists hold 16 more than
 // k, fewer where shared memory ends (a shorter slack only proves fewer queries).
@@ -1108,7 +1144,8 @@ bool tc_plan(long long n, long long nq, int d, int k, bool precise, int sms, TcP
   for (int most = kMaxCandTotal; most <= (precise ? 4 : 1) * kMaxCandTotal; most *= 2) {
     p->most_cand = most;
     p->share = tc_share(p->slab_rows, nq, p->cand, p->slabs, precise, most, sms);
-    int seg = p->share.max_segments();
+    p->equal = equal_if_exact(p->share, p->cand, most);
+    int seg = std::max(p->share.max_segments(), p->equal ? equal_segments(p->share) : 0);
     if (p->slabs > 1) {
       const TcShare last = tc_share(n - (long long)(p->slabs - 1) * p->slab_rows, nq, p->cand, p->slabs, precise, most, sms);
       seg = std::max(seg, last.max_segments());
@@ -1208,6 +1245,7 @@ cudaError_t run_tc(const TcPlan& p, const float* X, long long n, int d, const fl
     ta.seg0 = s * (p.nseg / p.slabs);
     ta.out = cand_buf;
     ta.inexact = xmax + 1;
+    ta.equal = p.equal;
     ta.err = err;
     bool fits = false;
     e = launch_tc<PRECISE, true, 8>(mq, mx, ta, maxsm, st, &fits);
