@@ -177,10 +177,10 @@ cudaError_t launch_edge_stats(const peos_codes_s* c, const float* q, int v, floa
 
 // brute force (knn.cu)
 size_t knn_scratch_bytes(int64_t n, int64_t nq, int k);
-// (qlist, qcount: device memory; only the listed queries from qfirst on, at most nq of them)
+// (qlist, qcount: device memory; only the listed queries, at most nq of them)
 cudaError_t launch_knn(const float* X, int64_t n, int d, const float* Q, int64_t nq, int k, int32_t* ids_out,
                        float* dists_out, void* scratch, cudaStream_t st, const int32_t* qlist = nullptr,
-                       const int* qcount = nullptr, int64_t qfirst = 0);
+                       const int* qcount = nullptr);
 
 // stage tracing (api.cu): while tracing is on, each search records events around its
 // stages (query tables, search kernel, re-rank) on its stream

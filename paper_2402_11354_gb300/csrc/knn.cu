@@ -8,9 +8,8 @@
 // writes them to scratch [nq][chunks][k].
 // Pass 2: one warp per query merges its chunks' lists into the final k.
 //
-// With a query list (`qlist`, its length in device memory) the same for up to nq of the listed
-// queries, from position `qfirst` on: the ones whose result the tensor-core form (knn_tc.cu)
-// could not prove.
+// With a query list (`qlist`, its length in device memory) the same for the listed queries
+// only: the ones whose result the tensor-core form (knn_tc.cu) could not prove.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -54,11 +53,8 @@ __global__ void __launch_bounds__(kThreads) knn_chunk_kernel(const float* __rest
                                                              const float* __restrict__ Q, long long nq, int k,
                                                              int nchunks, uint64_t* __restrict__ part,
                                                              const int32_t* __restrict__ qlist,
-                                                             const int* __restrict__ qcount, long long qfirst) {
-  if (qlist) {
-    nq = min(nq, *qcount - qfirst);
-    qlist += qfirst;
-  }
+                                                             const int* __restrict__ qcount) {
+  if (qlist) nq = *qcount;
   if ((long long)blockIdx.x * kQT >= nq) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* qs = reinterpret_cast<float*>(smem_raw);          // [kQT][kDK]
@@ -140,12 +136,8 @@ __global__ void __launch_bounds__(kThreads) knn_chunk_kernel(const float* __rest
 
 __global__ void knn_merge_kernel(const uint64_t* __restrict__ part, long long nq, int k, int nchunks,
                                  int32_t* __restrict__ ids_out, float* __restrict__ dists_out,
-                                 const int32_t* __restrict__ qlist, const int* __restrict__ qcount,
-                                 long long qfirst) {
-  if (qlist) {
-    nq = min(nq, *qcount - qfirst);
-    qlist += qfirst;
-  }
+                                 const int32_t* __restrict__ qlist, const int* __restrict__ qcount) {
+  if (qlist) nq = *qcount;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   uint64_t* lst = reinterpret_cast<uint64_t*>(smem_raw) + (size_t)warp * k;
@@ -183,7 +175,7 @@ size_t knn_scratch_bytes(int64_t n, int64_t nq, int k) {
 }
 
 cudaError_t launch_knn(const float* X, int64_t n, int d, const float* Q, int64_t nq, int k, int32_t* ids_out,
-                       float* dists_out, void* scratch, cudaStream_t st, const int32_t* qlist, const int* qcount, int64_t qfirst) {
+                       float* dists_out, void* scratch, cudaStream_t st, const int32_t* qlist, const int* qcount) {
   if (nq == 0) return cudaSuccess;
   const int nchunks = (int)((n + kChunk - 1) / kChunk);
   uint64_t* part = static_cast<uint64_t*>(scratch);
@@ -191,7 +183,7 @@ cudaError_t launch_knn(const float* X, int64_t n, int d, const float* Q, int64_t
   cudaError_t e = cudaFuncSetAttribute(knn_chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
   if (e != cudaSuccess) return e;
   dim3 grid1((unsigned)((nq + kQT - 1) / kQT), (unsigned)nchunks);
-  knn_chunk_kernel<<<grid1, kThreads, smem1, st>>>(X, n, d, Q, nq, k, nchunks, part, qlist, qcount, qfirst);
+  knn_chunk_kernel<<<grid1, kThreads, smem1, st>>>(X, n, d, Q, nq, k, nchunks, part, qlist, qcount);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int wpb = 4;
@@ -201,7 +193,7 @@ cudaError_t launch_knn(const float* X, int64_t n, int d, const float* Q, int64_t
   long long g2 = (nq + wpb - 1) / wpb;
   if (g2 > 65535) g2 = 65535;
   knn_merge_kernel<<<(unsigned)g2, wpb * 32, smem2, st>>>(part, nq, k, nchunks, ids_out, dists_out, qlist,
-                                                             qcount, qfirst);
+                                                             qcount);
   return cudaGetLastError();
 }
 
