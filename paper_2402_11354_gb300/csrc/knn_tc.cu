@@ -241,6 +241,8 @@ __global__ void convert_bf16_kernel(const float* __restrict__ X, long long n, in
       float s[kAtOnce];
 #pragma unroll
       for (int j = 0; j < kAtOnce; ++j) s[j] = 0.0f;
+      // two steps' loads in flight (1M x 128, 100 queries, the call: 505 us against 532; four 511)
+#pragma unroll 2
       for (int k = first + 4 * lane; k < end; k += 128) {
         float4 v[kAtOnce];
 #pragma unroll
@@ -298,15 +300,17 @@ __global__ void convert_bf16_kernel(const float* __restrict__ X, long long n, in
 struct TcShare {
   long long units;  // qt * bt
   int bt, G;
+  int Ge;           // CTAs of equal shares (G itself where the shares are not whole slices)
   int st, ns;       // tiles per slice, slices per query tile (st >= bt, 1: not sliced)
   int whole;
   __host__ __device__ long long start(int c, bool by_slices) const {
-    if (!by_slices) return units * c / G;
-    const long long s = units / bt * ns * c / G;  // the share's first slice
+    if (!by_slices) return units * min(c, Ge) / Ge;
+    const long long s = units / bt * ns * min(c, G) / G;  // the share's first slice
     return s / ns * bt + s % ns * st;
   }
   // the CTA whose share holds unit u (equal shares)
-  __host__ __device__ int cta_of(long long u) const { return (int)(((u + 1) * G - 1) / units); }
+  __host__ __device__ int cta_of(long long u) const { return (int)(((u + 1) * Ge - 1) / units); }
+  int ctas() const { return G > Ge ? G : Ge; }
   // the list of the segment of CTA c that ends with unit u, among its query tile's lists: from
   // one segment to the next the slice, the CTA or both go up
   __host__ __device__ int list_of(long long u, int c, long long cut, bool by_slices) const {
@@ -1044,7 +1048,7 @@ TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, i
   if (room >= 2) G = std::min(G, std::max(1LL, (room - 1) * qt));
   else G = std::min(G, qt);
   G = std::min(G, std::max(1LL, s.units / 4));
-  s.G = (int)std::max(1LL, G);
+  s.G = s.Ge = (int)std::max(1LL, G);
   if (s.ns > 1) {
     // whole slices where their uneven numbers cost less than the lists cut by equal shares
     const double start = list_tiles(256.0 * s.st, cand), slices = (double)(qt * s.ns);
@@ -1052,6 +1056,8 @@ TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, i
     if (room < 2 || ceil(slices / gw) * (s.st + start) <= (double)s.units / s.G + (slices / s.G + 1.0) * start) {
       s.whole = 1;
       s.G = gw;
+      // without slices
+      s.Ge = (int)std::max(1LL, std::min({(long long)sms, std::max(1LL, (most - 1) * qt), s.units / 4}));
     }
   }
   return s;
@@ -1059,17 +1065,18 @@ TcShare tc_share(long long n, long long nq, int cand, int slabs, bool precise, i
 
 // Whole slices are for scores that are rounded.  Where none is (the kernel finds out) a list goes
 // on past its slice, and equal shares are taken after all if the CTA that has most to do then has
-// less (606,000 x 128 integer rows, 11,863 queries, k = 1: 1,580 tiles at most against 1,449,
-// 3,227 us against 3,033; 6,900 rows, 3,838 queries, k = 27 keep the slices, where a CTA
-// starts one list and not two: 406 us, 577 with equal shares).
+// less: its tiles and its lists' insertions, each about 1.2 tiles' time (integer rows of 128:
+// 606,000, 11,863 queries, k = 1 1,580 tiles at most against 1,449, 3,227 us against 3,033;
+// 314,000, 6,681 queries, k = 1 614 tiles and one list against 428 and two, 1,399 us against 1,336).
 double busiest(const TcShare& s, bool by_slices, int cand) {
   double most = 0.0;
-  for (int c = 0; c < s.G; ++c) {
+  for (int c = 0; c < s.ctas(); ++c) {
     const long long u1 = s.start(c + 1, by_slices);
     double cost = 0.0;
     for (long long u = s.start(c, by_slices); u < u1;) {
       const long long ue = std::min(u1, (u / s.bt + 1) * s.bt);
-      cost += (double)(ue - u) + list_tiles(256.0 * (ue - u), cand);
+      const double rows = 256.0 * (ue - u);
+      cost += (double)(ue - u) + 1.2 * cand * (rows > cand ? 1.0 + log(rows / cand) : 1.0);
       u = ue;
     }
     most = std::max(most, cost);
@@ -1083,10 +1090,10 @@ int equal_segments(TcShare s) {
 }
 int equal_if_exact(const TcShare& s, int cand, int most_cand) {
   // looked at where the slices' uneven numbers cost 4% of at least 256 tiles a CTA (the sums
-  // below take some 8 us of the host)
-  const long long slices = s.units / s.bt * s.ns, least = (s.units + s.G - 1) / s.G;
-  if (least < 256 || (slices + s.G - 1) / s.G * s.st * 100 < least * 104) return 0;
-  return s.whole && equal_segments(s) * cand <= most_cand && busiest(s, false, cand) < busiest(s, true, cand);
+  // take some 8 us of the host)
+  const long long slices = s.units / s.bt * s.ns, least = (s.units + s.Ge - 1) / s.Ge;
+  if (!s.whole || least < 256 || (slices + s.G - 1) / s.G * s.st * 100 < least * 104) return 0;
+  return equal_segments(s) * cand <= most_cand && busiest(s, false, cand) < busiest(s, true, cand);
 }
 
 // The longest list whose launch fits in shared memory (4 epilogue warps, two stages of query
@@ -1197,7 +1204,7 @@ cudaError_t launch_tc(const CUtensorMap& mq, const CUtensorMap& mx, TcArgs ta, i
   ta.stages = stages;
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  fn<<<(unsigned)ta.share.G, (EW + 2) * 32, smem, st>>>(mq, mx, ta);
+  fn<<<(unsigned)ta.share.ctas(), (EW + 2) * 32, smem, st>>>(mq, mx, ta);
   return cudaGetLastError();
 }
 
