@@ -12,13 +12,14 @@
 //      mbarriers (the query chunks stay resident where they fit); an MMA warp issues
 //      tcgen05.mma (BF16 in, FP32 accumulate in tensor memory, M = 128, N = 256, K = 16 per
 //      instruction) into one of two accumulators, in the precise form for the products hi hi,
-//      lo hi and hi lo; four epilogue warps read the other accumulator with tcgen05.ld, one
-//      query row per thread, and keep the row's best `cand` scores ||x||^2 - 2 q.x (q's own
-//      norm does not change the order) in a max-heap in shared memory.  Scores below the
-//      heap's worst wait in a short per-row buffer; when a row's buffer is nearly full all
-//      rows empty theirs side by side.
+//      lo hi and hi lo; eight epilogue warps (four where the lists are long) read the other
+//      accumulator with tcgen05.ld, one query row per thread, and keep the row's best `cand`
+//      scores ||x||^2 - 2 q.x (q's own norm does not change the order) in a max-heap in shared
+//      memory.  Scores below the heap's worst wait in a short per-row buffer; when a row's
+//      buffer is nearly full all rows empty theirs side by side.
 //      Where scores are rounded the plain form closes a list at the end of a slice of the base
-//      too, so that a query keeps as many rows as it takes to absorb misranked ones.
+//      too, so that a query keeps as many rows as it takes to absorb misranked ones, and the
+//      CTAs take whole slices where that costs less.
 //   3. finalize: the candidates of every segment sorted by score; those that may be among
 //      the k nearest (score within twice the error bound of the k-th) get their exact FP32
 //      squared distance (sequential over the dimensions), and the k smallest by (dist, id)
@@ -30,7 +31,8 @@
 //
 // The precise form proves its result: a row left out of a full list scored no better than
 // that list's worst, so with the score's error bound its distance is known to be above
-// the k-th found, or the query is handed on to the FFMA kernel (knn.cu).  Norms that vanish
+// the k-th found (rows too long to be near the query aside, whatever their error), or the
+// query is handed on to the FFMA kernel (knn.cu).  Norms that vanish
 // or come near FP32's range and a CTA that gave up waiting hand every query on.
 //
 // Every wait on an mbarrier is bounded: after kWaitLimitNs of the global timer (or
